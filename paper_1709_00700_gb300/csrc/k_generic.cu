@@ -7,10 +7,11 @@
 // (whose row count exists only on the device), or when the variant asks for
 // them (pv_variant.interp = 1).
 //
-// One thread takes one row at a time, grid-stride over rows, so neighbouring
-// lanes read neighbouring rows of each column (coalesced scalar loads).
-// Branched mode stops at a row's first failing operation; predicated mode
-// evaluates every predicate and probe of every row (Section 6).  The sinks
+// The aggregations take U items (of 4 consecutive rows) per thread through
+// each operation together; the projections and the key pass take one row at a
+// time, grid-stride over rows.  Branched mode stops at a row's (an item's)
+// first failing operation; predicated mode evaluates every predicate and
+// probe of every row (Section 6).  The sinks
 // are those of the compiled kernels with the aggregate functions read at run
 // time: AGGREGATE with per-thread accumulators and one atomic per CTA and
 // aggregate; PROJECT single pass (warp-aggregated atomics) or multi pass
@@ -79,23 +80,6 @@ __device__ __forceinline__ int64_t g_ref(const KParams& kp, const GenSpec& gs, c
   return static_cast<int32_t>(gload(gs.pay_col[x.a][x.b], gs.pay_type[x.a][x.b], b));
 }
 
-// ARITHMETIC: the product of the aggregate's terms, wrapping int64 (COUNT: 1).
-__device__ __forceinline__ int64_t g_value(const KParams& kp, const GenSpec& gs, const GAgg& a, int64_t r,
-                                           const int32_t (&bind)[PV_MAX_PROBES]) {
-  if (a.func == PV_COUNT) return 1;
-  uint64_t v = 1;
-#pragma unroll
-  for (int t = 0; t < PV_MAX_TERMS; ++t) {
-    if (t < a.n_terms) {
-      const GTerm& m = a.t[t];
-      const uint64_t x = static_cast<uint64_t>(g_ref(kp, gs, m.x, r, bind));
-      const uint64_t c = static_cast<uint64_t>(m.c);
-      v *= m.kind == PV_TERM_X ? x : m.kind == PV_TERM_X_PLUS_C ? x + c : c - x;
-    }
-  }
-  return static_cast<int64_t>(v);
-}
-
 // Accumulator codes (MIN/MAX as order-preserving codes, so that every word
 // starts at 0 and merges with add or max).
 __device__ __forceinline__ bool is_minmax(int f) { return f == PV_MIN || f == PV_MAX; }
@@ -109,36 +93,249 @@ __device__ __forceinline__ uint64_t g_warp_reduce(int f, uint64_t v) {
   return is_minmax(f) ? warp_reduce<PV_MAX>(v) : warp_reduce<PV_SUM>(v);
 }
 
-// Codes of one surviving row: c[a] for the aggregates, c[PV_MAX_AGGS] = 1.
-__device__ __forceinline__ void g_codes(const KParams& kp, const GenSpec& gs, int64_t r,
-                                        const int32_t (&bind)[PV_MAX_PROBES], uint64_t (&c)[kGW]) {
+// ---------------------------------------------------------------------------
+// Evaluation by items.  A thread takes U items of 4 consecutive rows through
+// one operation at a time, so that the loads of one operation are all in
+// flight together (U 16-byte loads of an int32 column) and the run-time
+// dispatch on the program is paid once per 4 * U rows.  One row at a time,
+// these kernels were bound by the latency of one row's chain of dependent
+// loads: 30M rows of three filters and a product took 426 us (27% of the
+// bytes' time at the copy rate went to DRAM), 20M rows of two probes 353 us.
+// What the probes bind is indexed by the probe number at run time, so it
+// lives in local memory (16-byte stores and loads that stay in L1).
+// ---------------------------------------------------------------------------
+constexpr int kGUAgg = 2;    // items per thread, AGGREGATE: 30M rows 426 -> 158 us
+constexpr int kGUGroup = 2;  // items per thread, HASH_AGGREGATE: 20M rows, two probes 353 -> 190 us
+
+template <int U>
+struct GItems {
+  int64_t item[U];
+  int n[U];          // rows of the item inside the table, 0..4
+  uint32_t mask[U];  // surviving rows
+};
+
+// The 4 rows of an item; vec: the column starts on a 16-byte boundary (result
+// columns of an earlier grouped pipeline may not).
+template <class T>
+__device__ __forceinline__ void g_load4(T (&d)[4], const void* base, int64_t item, int n, bool vec) {
+  const T* p = static_cast<const T*>(base) + item * 4;
+  if (n == 4 && vec) {
+    if constexpr (sizeof(T) == 4) {
+      const int4 q = __ldg(reinterpret_cast<const int4*>(p));
+      d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
+    } else if constexpr (sizeof(T) == 8) {
+      const longlong2 a = __ldg(reinterpret_cast<const longlong2*>(p));
+      const longlong2 b = __ldg(reinterpret_cast<const longlong2*>(p) + 1);
+      d[0] = a.x; d[1] = a.y; d[2] = b.x; d[3] = b.y;
+    } else {
+      const uchar4 q = __ldg(reinterpret_cast<const uchar4*>(p));
+      d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
+    }
+  } else {
 #pragma unroll
-  for (int a = 0; a < PV_MAX_AGGS; ++a)
-    c[a] = a < gs.n_aggs ? g_code(gs.agg[a].func, g_value(kp, gs, gs.agg[a], r, bind)) : 0;
-  c[PV_MAX_AGGS] = 1;
+    for (int r = 0; r < 4; ++r) d[r] = r < n ? __ldg(p + r) : T(0);
+  }
+}
+
+__device__ __forceinline__ bool g_aligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+// Column values of the items in `need` (bit u: item u) as int64.
+template <class T, int U>
+__device__ __forceinline__ void g_items_as(int64_t (&v)[U][4], const void* base, const GItems<U>& it, uint32_t need) {
+  T d[U][4];
+  const bool vec = g_aligned(base);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if ((need >> u) & 1u) {
+      g_load4<T>(d[u], base, it.item[u], it.n[u], vec);
+    } else {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) d[u][r] = T(0);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[u][r] = static_cast<int64_t>(d[u][r]);
+}
+template <int U>
+__device__ __forceinline__ void g_items_col(int64_t (&v)[U][4], const void* base, int type, const GItems<U>& it,
+                                            uint32_t need) {
+  if (type == PV_I32) g_items_as<int32_t, U>(v, base, it, need);
+  else if (type == PV_I64) g_items_as<int64_t, U>(v, base, it, need);
+  else g_items_as<uint8_t, U>(v, base, it, need);
+}
+
+// Items whose columns an operation reads: those with a live row, or in
+// predicated mode those with a row.
+template <int U>
+__device__ __forceinline__ uint32_t g_need(const GItems<U>& it, bool pred) {
+  uint32_t need = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) need |= static_cast<uint32_t>(pred ? it.n[u] > 0 : it.mask[u] != 0) << u;
+  return need;
+}
+
+// What the probes bound, by probe, item and row.
+template <int U>
+struct GBind {
+  int4 v[PV_MAX_PROBES][U];
+};
+
+// FILTER and HASH_PROBE of the items, in the program's order.
+template <int U>
+__device__ __forceinline__ void g_eval_items(const KParams& kp, const GenSpec& gs, GItems<U>& it, bool pred,
+                                             GBind<U>& bind) {
+#pragma unroll 1
+  for (int i = 0; i < gs.n_preds; ++i) {
+    const uint32_t need = g_need<U>(it, pred);
+    if (need == 0) return;
+    const int s = gs.pred_slot[i];
+    const int64_t lo = kp.lo[i], hi = kp.hi[i];
+    int64_t v[U][4];
+    g_items_col<U>(v, kp.col[s], gs.slot_type[s], it, need);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      uint32_t b = 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) b |= static_cast<uint32_t>((v[u][r] >= lo) & (v[u][r] <= hi)) << r;
+      it.mask[u] &= b;
+    }
+  }
+#pragma unroll 1
+  for (int j = 0; j < gs.n_probes; ++j) {
+    const uint32_t need = g_need<U>(it, pred);
+    if (need == 0) return;
+    const int s = gs.probe_slot[j];
+    const DevHT& h = kp.probe[j];
+    int64_t k[U][4];
+    g_items_col<U>(k, kp.col[s], gs.slot_type[s], it, need);
+    const bool wide = gs.slot_type[s] == PV_I64;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      int32_t pay[4] = {0, 0, 0, 0};
+      if ((need >> u) & 1u) {
+        if (wide) {
+          it.mask[u] = probe_item(h, k[u], it.mask[u], pay, pred && it.n[u] == 4);
+        } else {
+          int32_t k32[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) k32[r] = static_cast<int32_t>(k[u][r]);
+          it.mask[u] = probe_item(h, k32, it.mask[u], pay, pred && it.n[u] == 4);
+        }
+      }
+      bind.v[j][u] = make_int4(pay[0], pay[1], pay[2], pay[3]);
+    }
+  }
+}
+
+// Values of a reference for the live rows of the items (0 elsewhere, or what
+// the rest of a loaded item holds).
+template <int U>
+__device__ __forceinline__ void g_items_ref(const KParams& kp, const GenSpec& gs, const GRef& x, const GItems<U>& it,
+                                            const GBind<U>& bind, int64_t (&v)[U][4]) {
+  if (x.kind == PV_REF_COL) {
+    g_items_col<U>(v, kp.col[x.a], gs.slot_type[x.a], it, g_need<U>(it, false));
+    return;
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int4 b = bind.v[x.a][u];
+    v[u][0] = b.x; v[u][1] = b.y; v[u][2] = b.z; v[u][3] = b.w;
+  }
+  if (gs.indexed[x.a]) {
+    const void* col = gs.pay_col[x.a][x.b];
+    const int type = gs.pay_type[x.a][x.b];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        v[u][r] = (it.mask[u] >> r) & 1u ? static_cast<int32_t>(gload(col, type, v[u][r])) : 0;
+  }
+}
+
+// ARITHMETIC for the live rows of the items: the product of the aggregate's
+// terms, wrapping int64 (COUNT: 1).
+template <int U>
+__device__ __forceinline__ void g_items_value(const KParams& kp, const GenSpec& gs, const GAgg& a,
+                                              const GItems<U>& it, const GBind<U>& bind, int64_t (&v)[U][4]) {
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[u][r] = 1;
+  if (a.func == PV_COUNT) return;
+#pragma unroll 1
+  for (int t = 0; t < a.n_terms; ++t) {
+    const GTerm& m = a.t[t];
+    int64_t x[U][4];
+    g_items_ref<U>(kp, gs, m.x, it, bind, x);
+    // x, x + c and c - x as add + sign * x
+    const uint64_t add = m.kind == PV_TERM_X ? 0 : static_cast<uint64_t>(m.c);
+    const bool neg = m.kind == PV_TERM_C_MINUS_X;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const uint64_t y = static_cast<uint64_t>(x[u][r]);
+        v[u][r] = static_cast<int64_t>(static_cast<uint64_t>(v[u][r]) * (add + (neg ? 0ull - y : y)));
+      }
+  }
+}
+
+// Grid-stride loop over groups of U items (thread t: items t, t + T, ... of a
+// trip, so neighbouring lanes read neighbouring items).
+template <int U, class F>
+__device__ __forceinline__ void g_for_items(int64_t n, F&& f) {
+  const int64_t n_items = (n + 3) >> 2;
+  const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; base < n_items; base += U * T) {
+    GItems<U> it;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      it.item[u] = base + u * T;
+      const int64_t left = n - it.item[u] * 4;
+      it.n[u] = left >= 4 ? 4 : (left > 0 ? static_cast<int>(left) : 0);
+      it.mask[u] = (1u << it.n[u]) - 1u;
+    }
+    f(it);
+  }
 }
 
 // ---------------------------------------------------------------------------
 // AGGREGATE
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_gen_aggregate(const __grid_constant__ KParams kp,
+__global__ void __maxnreg__(64) k_gen_aggregate(const __grid_constant__ KParams kp,
                                                         const __grid_constant__ GenSpec gs,
                                                         const __grid_constant__ AggOut out, int pred) {
   uint64_t acc[kGW];
 #pragma unroll
   for (int a = 0; a < kGW; ++a) acc[a] = 0;
-  const int64_t n = g_rows(kp, gs);
-  for (int64_t r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; r < n;
-       r += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    int32_t bind[PV_MAX_PROBES];
-    if (!g_row(kp, gs, r, pred != 0, bind)) continue;
-    uint64_t c[kGW];
-    g_codes(kp, gs, r, bind, c);
+  g_for_items<kGUAgg>(g_rows(kp, gs), [&](GItems<kGUAgg>& it) {
+    GBind<kGUAgg> bind;
+    g_eval_items<kGUAgg>(kp, gs, it, pred != 0, bind);
+    uint32_t live = 0;
 #pragma unroll
-    for (int a = 0; a < PV_MAX_AGGS; ++a)
-      if (a < gs.n_aggs) acc[a] = g_combine(gs.agg[a].func, acc[a], c[a]);
-    acc[PV_MAX_AGGS] += 1;
-  }
+    for (int u = 0; u < kGUAgg; ++u) live += __popc(it.mask[u]);
+    if (live == 0) return;
+    acc[PV_MAX_AGGS] += live;
+#pragma unroll 1
+    for (int a = 0; a < gs.n_aggs; ++a) {
+      const int f = gs.agg[a].func;
+      if (f == PV_COUNT) {
+        acc[a] += live;
+        continue;
+      }
+      int64_t v[kGUAgg][4];
+      g_items_value<kGUAgg>(kp, gs, gs.agg[a], it, bind, v);
+      uint64_t c = 0;  // of the trip's rows: one update of acc[a], which lives in local memory
+#pragma unroll
+      for (int u = 0; u < kGUAgg; ++u)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if ((it.mask[u] >> r) & 1u) c = g_combine(f, c, g_code(f, v[u][r]));
+      acc[a] = g_combine(f, acc[a], c);
+    }
+  });
   // CTA epilogue: warp shuffles, one slot per warp, one atomic per word; the
   // last CTA decodes the result and re-zeroes the accumulators.
   __shared__ unsigned long long red[32][kGW];
@@ -363,92 +560,177 @@ __device__ __forceinline__ void g_key(const KParams& kp, const GenSpec& gs, cons
   else packed = (static_cast<uint64_t>(static_cast<uint32_t>(part[0])) << 32) | static_cast<uint32_t>(part[1]);
 }
 
-// Adds one row's codes (or a local table's slot) into a slot: SUM/COUNT add,
-// MIN/MAX take the max of codes; the row count goes to word n_aggs only when
-// no COUNT aggregate holds it.  SHARED: the slot is in shared memory.
+// One accumulator word: SUM/COUNT add, MIN/MAX take the max of codes (only
+// when the word is smaller: most rows of a group raise neither).  SHARED: the
+// word is in shared memory.
 template <bool SHARED>
-__device__ __forceinline__ void g_slot_add(unsigned long long* v, const uint64_t (&c)[kGW], const GroupDesc& gd) {
-#pragma unroll
-  for (int a = 0; a < PV_MAX_AGGS; ++a) {
-    if (a < gd.n_aggs && c[a] != 0) {
-      if (is_minmax(gd.func[a])) atomicMax(v + a, static_cast<unsigned long long>(c[a]));
-      else if constexpr (SHARED) shared_add64(v + a, c[a]);
-      else atomicAdd(v + a, static_cast<unsigned long long>(c[a]));
+__device__ __forceinline__ void g_word_add(unsigned long long* w, int f, uint64_t c) {
+  if (c == 0) return;
+  if (is_minmax(f)) {
+    if constexpr (SHARED) {
+      if (*reinterpret_cast<volatile unsigned long long*>(w) >= c) return;
     }
-  }
-  if (gd.count_word == gd.n_aggs && c[PV_MAX_AGGS] != 0) {
-    if constexpr (SHARED) shared_add64(v + gd.n_aggs, c[PV_MAX_AGGS]);
-    else atomicAdd(v + gd.n_aggs, static_cast<unsigned long long>(c[PV_MAX_AGGS]));
+    atomicMax(w, static_cast<unsigned long long>(c));
+  } else if constexpr (SHARED) {
+    shared_add64(w, c);
+  } else {
+    atomicAdd(w, static_cast<unsigned long long>(c));
   }
 }
 
+// Copies of a CTA-local perfect array of `words` words: lane l adds into copy
+// l % R, word w of copy c at smem[w * R + c].  With few groups the lanes of a
+// warp meet in the same words, and same-word shared atomics take turns; copies
+// within 32 KB leave the SM's other CTAs their share.
+constexpr int kGCopiesBytes = 32 << 10;
+__host__ __device__ inline int g_local_copies(int64_t words) {
+  int r = 32;
+  while (r > 1 && words * r * 8 > kGCopiesBytes) r >>= 1;
+  return r;
+}
+
 template <int SK, int GM>
-__global__ void __launch_bounds__(1024) k_gen_group(const __grid_constant__ KParams kp,
-                                                    const __grid_constant__ GenSpec gs,
-                                                    const __grid_constant__ GroupDesc gd,
-                                                    const __grid_constant__ GroupOut g, int pred) {
+__global__ void __maxnreg__(64) k_gen_group(const __grid_constant__ KParams kp,
+                                            const __grid_constant__ GenSpec gs,
+                                            const __grid_constant__ GroupDesc gd,
+                                            const __grid_constant__ GroupOut g, int pred) {
+  constexpr int U = kGUGroup;
   extern __shared__ unsigned long long smem[];
   if (blockIdx.x == 0 && threadIdx.x == 0) *g.out_count = 0;  // extraction runs after this kernel
   unsigned long long* lk = smem;                               // local hash table: keys, then values
   unsigned long long* lv = smem + (SK == GS_LOCAL_HASH ? g.local_slots : 0);
+  const int R = SK == GS_LOCAL_PERFECT ? g_local_copies(g.cap * g.stride) : 1;  // copies of the local table
   if constexpr (SK == GS_LOCAL_PERFECT) {
-    for (int64_t i = threadIdx.x; i < g.cap * g.stride; i += blockDim.x) smem[i] = 0;
+    for (int64_t i = threadIdx.x; i < g.cap * g.stride * R; i += blockDim.x) smem[i] = 0;
     __syncthreads();
   } else if constexpr (SK == GS_LOCAL_HASH) {
     for (int i = threadIdx.x; i < g.local_slots; i += blockDim.x) lk[i] = kEmpty64;
     for (int64_t i = threadIdx.x; i < static_cast<int64_t>(g.local_slots) * g.stride; i += blockDim.x) lv[i] = 0;
     __syncthreads();
   }
-  const int64_t n = g_rows(kp, gs);
   unsigned long long* rep = g.vals + (blockIdx.x % g.replicas) * g.rep_stride;
-  for (int64_t r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; r < n;
-       r += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    int32_t bind[PV_MAX_PROBES];
-    if (!g_row(kp, gs, r, pred != 0, bind)) continue;
-    uint64_t code, key;
-    bool in_domain;
-    g_key(kp, gs, gd, r, bind, code, key, in_domain);
-    if (!in_domain && (SK == GS_GLOBAL_PERFECT || SK == GS_LOCAL_PERFECT || gd.coded)) {
-      set_error(kp.err, PV_ERR_KEY_OUT_OF_RANGE);
-      continue;
+  const int copy = SK == GS_LOCAL_PERFECT ? static_cast<int>(threadIdx.x) & (R - 1) : 0;
+  g_for_items<U>(g_rows(kp, gs), [&](GItems<U>& it) {
+    GBind<U> bind;
+    g_eval_items<U>(kp, gs, it, pred != 0, bind);
+    if (g_need<U>(it, false) == 0) return;
+    // Key of each live row: the mixed-radix code of its parts over their
+    // domains (the perfect-array slot, and the hash key of coded keys), else
+    // the packed key (one part, or two 32-bit halves).
+    constexpr bool kPerfect = SK == GS_GLOBAL_PERFECT || SK == GS_LOCAL_PERFECT;
+    const bool coded = kPerfect || gd.coded;
+    const bool whole = gs.n_keys == 1 && gd.key64[0];
+    uint64_t key[U][4];
+    uint32_t in_domain[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      in_domain[u] = 0xFu;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) key[u][r] = 0;
     }
-    uint64_t c[kGW];
-    g_codes(kp, gs, r, bind, c);
-    if constexpr (SK == GS_GLOBAL_PERFECT) {
-      g_slot_add<false>(rep + code * g.stride, c, gd);
-    } else if constexpr (SK == GS_LOCAL_PERFECT) {
-      g_slot_add<true>(smem + code * g.stride, c, gd);
-    } else {
-      if constexpr (SK == GS_LOCAL_HASH) {
-        if (key != kEmpty64) {
-          const uint32_t mask = static_cast<uint32_t>(g.local_slots) - 1;
-          uint32_t idx = static_cast<uint32_t>(fmix64(key)) & mask;
-          bool placed = false;
-          for (int step = 0; step < kLocalProbe && !placed; ++step) {
-            unsigned long long cur = *reinterpret_cast<volatile unsigned long long*>(lk + idx);
-            if (cur == kEmpty64) cur = atomicCAS(lk + idx, kEmpty64, static_cast<unsigned long long>(key));
-            if (cur == kEmpty64 || cur == key) {
-              g_slot_add<true>(lv + static_cast<uint64_t>(idx) * g.stride, c, gd);
-              placed = true;
-            }
-            idx = (idx + 1) & mask;
+#pragma unroll 1
+    for (int i = 0; i < gs.n_keys; ++i) {
+      int64_t part[U][4];
+      g_items_ref<U>(kp, gs, gs.key[i], it, bind, part);
+      const uint64_t mn = static_cast<uint64_t>(gd.key_min[i]), span = static_cast<uint64_t>(gd.key_span[i]);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const uint64_t p = static_cast<uint64_t>(part[u][r]);
+          if (coded) {
+            if (p - mn >= span) in_domain[u] &= ~(1u << r);
+            key[u][r] = key[u][r] * span + (p - mn);
+          } else {
+            key[u][r] = whole ? p : (key[u][r] << 32) | static_cast<uint32_t>(p);
           }
-          if (placed) continue;
+        }
+    }
+    // Slot of each live row (in key[][] from here on); rows without one leave
+    // the mask.  Hash tables take the rows one by one (their probe sequences
+    // differ), with the keys in local memory.
+    uint32_t live = 0, slot_local = 0;  // bit 4u + r; slot_local: the row's slot is in the local table
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (it.mask[u] & ~in_domain[u]) set_error(kp.err, PV_ERR_KEY_OUT_OF_RANGE);
+      live |= (it.mask[u] & in_domain[u]) << (4 * u);
+    }
+    if constexpr (!kPerfect) {
+#pragma unroll 1
+      for (uint32_t todo = live; todo != 0; todo &= todo - 1) {
+        const int i = __ffs(todo) - 1;
+        const uint64_t k = key[i >> 2][i & 3];
+        bool placed = false;
+        if constexpr (SK == GS_LOCAL_HASH) {
+          if (k != kEmpty64) {
+            const uint32_t mask = static_cast<uint32_t>(g.local_slots) - 1;
+            uint32_t idx = static_cast<uint32_t>(fmix64(k)) & mask;
+            for (int step = 0; step < kLocalProbe && !placed; ++step) {
+              unsigned long long cur = *reinterpret_cast<volatile unsigned long long*>(lk + idx);
+              if (cur == kEmpty64) cur = atomicCAS(lk + idx, kEmpty64, static_cast<unsigned long long>(k));
+              if (cur == kEmpty64 || cur == k) {
+                key[i >> 2][i & 3] = idx;
+                slot_local |= 1u << i;
+                placed = true;
+              }
+              idx = (idx + 1) & mask;
+            }
+          }
+        }
+        if (!placed) {  // rows that found no local slot, too
+          const uint64_t s = global_slot<GM>(g, k, kp.err);
+          key[i >> 2][i & 3] = s;
+          if (s > static_cast<uint64_t>(g.cap)) live &= ~(1u << i);
         }
       }
-      const uint64_t s = global_slot<GM>(g, key, kp.err);  // rows that found no local slot, too
-      if (s <= static_cast<uint64_t>(g.cap)) g_slot_add<false>(g.vals + s * g.stride, c, gd);
     }
-  }
+#pragma unroll
+    for (int u = 0; u < U; ++u) it.mask[u] = (live >> (4 * u)) & 0xFu;
+    // Word a of each live row's slot; the row count goes to word n_aggs only
+    // when no COUNT aggregate holds it.
+    auto add_word = [&](int a, int f, const int64_t (&v)[U][4]) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (!((it.mask[u] >> r) & 1u)) continue;
+          const uint64_t c = g_code(f, v[u][r]);
+          const uint64_t w = key[u][r] * g.stride + a;
+          if constexpr (SK == GS_LOCAL_PERFECT) {
+            g_word_add<true>(smem + w * R + copy, f, c);
+          } else if constexpr (SK == GS_GLOBAL_PERFECT) {
+            g_word_add<false>(rep + w, f, c);
+          } else if constexpr (SK == GS_LOCAL_HASH) {
+            if ((slot_local >> (4 * u + r)) & 1u) g_word_add<true>(lv + w, f, c);
+            else g_word_add<false>(g.vals + w, f, c);
+          } else {
+            g_word_add<false>(g.vals + w, f, c);
+          }
+        }
+    };
+    int64_t v[U][4];
+#pragma unroll 1
+    for (int a = 0; a < gd.n_aggs; ++a) {
+      g_items_value<U>(kp, gs, gs.agg[a], it, bind, v);
+      add_word(a, gd.func[a], v);
+    }
+    if (gd.count_word == gd.n_aggs) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[u][r] = 1;
+      add_word(gd.n_aggs, PV_COUNT, v);
+    }
+  });
   pdl_launch_dependents();  // the extraction kernel may start launching now
   if constexpr (SK == GS_LOCAL_PERFECT) {
     __syncthreads();
     for (int64_t i = threadIdx.x; i < g.cap * g.stride; i += blockDim.x) {
-      const uint64_t v = smem[i];
-      if (!v) continue;
       const int a = static_cast<int>(i % g.stride);
-      if (a < gd.n_aggs && is_minmax(gd.func[a])) atomicMax(rep + i, static_cast<unsigned long long>(v));
-      else atomicAdd(rep + i, static_cast<unsigned long long>(v));
+      const int f = a < gd.n_aggs ? gd.func[a] : PV_SUM;
+      uint64_t v = 0;
+      for (int k = 0; k < R; ++k) v = g_combine(f, v, smem[i * R + ((k + threadIdx.x) & (R - 1))]);
+      g_word_add<false>(rep + i, f, v);
     }
   } else if constexpr (SK == GS_LOCAL_HASH) {
     __syncthreads();
@@ -456,13 +738,11 @@ __global__ void __launch_bounds__(1024) k_gen_group(const __grid_constant__ KPar
       const uint64_t key = lk[i];
       if (key == kEmpty64) continue;
       const unsigned long long* w = lv + static_cast<uint64_t>(i) * g.stride;
-      uint64_t c[kGW];
-#pragma unroll
-      for (int a = 0; a < PV_MAX_AGGS; ++a) c[a] = a < gd.n_aggs ? w[a] : 0;
-      c[PV_MAX_AGGS] = gd.count_word == gd.n_aggs ? w[gd.n_aggs] : 0;
       if (w[gd.count_word] == 0) continue;
       const uint64_t s = global_slot<GM>(g, key, kp.err);
-      if (s <= static_cast<uint64_t>(g.cap)) g_slot_add<false>(g.vals + s * g.stride, c, gd);
+      if (s > static_cast<uint64_t>(g.cap)) continue;
+      for (int a = 0; a <= gd.n_aggs; ++a)
+        g_word_add<false>(g.vals + s * g.stride + a, a < gd.n_aggs ? gd.func[a] : PV_SUM, w[a]);
     }
   }
 }
@@ -555,8 +835,9 @@ pv_status generic_grouped(const LaunchCfg& c, const KParams& kp, const GenSpec& 
   if (g.ht == PV_HT_PERFECT) {
     if (multi) return PV_ERR_UNSUPPORTED;  // no keys to insert
     if (local) {
-      const size_t smem = static_cast<size_t>(g.cap) * slot_bytes;
+      size_t smem = static_cast<size_t>(g.cap) * slot_bytes;
       if (smem > kLocalPerfectBytes) return PV_ERR_UNSUPPORTED;
+      smem *= g_local_copies(g.cap * g.stride);
       s = g_launch(c, k_gen_group<GS_LOCAL_PERFECT, G_INSERT>, smem, kp.n_rows, kp, gs, gd, g, pred);
     } else {
       s = g_launch(c, k_gen_group<GS_GLOBAL_PERFECT, G_INSERT>, 0, kp.n_rows, kp, gs, gd, g, pred);
