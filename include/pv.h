@@ -166,7 +166,7 @@ typedef enum { PV_GRID_STRIDE = 0, PV_CHUNKED = 1, PV_STAGED = 2 } pv_access;
 
 typedef struct {
   int32_t exec;              /* pv_exec: projection single pass (warp-aggregated atomics) or
-                                count -> prefix sum -> scatter; aggregation: fused, or keys first */
+                                ordered by a prefix sum of match counts; aggregation: fused, or keys first */
   int32_t agg;               /* pv_agg_strategy for HASH_AGGREGATE */
   int32_t pred;              /* pv_pred_mode (all operations of the pipeline share it) */
   int32_t access;            /* pv_access: coalesced grid-stride, per-thread chunks, or TMA-staged chunks */
@@ -462,7 +462,7 @@ pv_status pv_mlp_adam(pv_ctx* ctx, float* params, const float* grad, float* m, f
  * has reserved the device), and latency-critical code that cannot pay for
  * cudaMalloc's device-wide synchronisation.  It needs no pv_ctx.
  *
- * Computes the multi-pass projection (count -> prefix sum -> scatter, as
+ * Computes the multi-pass projection (ordered by a prefix sum of match counts, as
  * pv_run_pipeline with PV_EXEC_MULTI_PASS) of
  *     SELECT a, price FROM t WHERE a_lo <= a <= a_hi AND b_lo <= b <= b_hi
  * over n_rows rows of the int32 columns a, b and the int64 column price
@@ -472,8 +472,8 @@ pv_status pv_mlp_adam(pv_ctx* ctx, float* params, const float* grad, float* m, f
  * out_capacity) and *out_status (device int32) = PV_OK, or
  * PV_ERR_OUTPUT_OVERFLOW when more rows matched than fit.
  *
- * It allocates nothing: its scratch (an error word plus per-tile counts and
- * offsets, about 1 MB) is one statically sized array in device memory that
+ * It allocates nothing: its scratch (an error word, a ticket and one word per
+ * tile, about 0.5 MB) is one statically sized array in device memory that
  * every GPU loading this library holds until the process exits.  The first
  * call on a device, with that device current, looks up the array's device
  * address (cudaGetSymbolAddress) and caches it; make that first call before

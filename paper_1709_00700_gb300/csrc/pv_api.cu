@@ -643,16 +643,22 @@ static pv_status alloc_result(pv_ctx* c, Result& r) {
     const int block = r.var.block ? r.var.block : 256;
     const int64_t tile_items = static_cast<int64_t>(block) * U;
     r.proj.n_tiles = std::max<int64_t>(1, (k.kp.n_items + tile_items - 1) / tile_items);
-    const size_t ctl = 32 + 16 * static_cast<size_t>(r.var.exec == PV_EXEC_MULTI_PASS ? r.proj.n_tiles : 0);
-    char* p = static_cast<char*>(grab(ctl));
+    const bool multi = r.var.exec == PV_EXEC_MULTI_PASS;
+    const size_t scratch = !multi ? 0 : r.generic ? 16 * static_cast<size_t>(r.proj.n_tiles) : mark_bytes(k.n_rows);
+    const size_t ctl = 32 + (multi && r.generic ? scratch : 0);  // zeroed here; the marks are cleared by each run
+    char* p = static_cast<char*>(grab(32 + scratch));
     if (!p) return fail(c, PV_ERR_OOM, "allocator returned NULL");
     PV_CUDA(c, cudaMemsetAsync(p, 0, ctl, c->stream));
     r.proj.cursor = reinterpret_cast<unsigned long long*>(p);
     r.proj.count = reinterpret_cast<int64_t*>(p + 8);
     r.proj.done = reinterpret_cast<unsigned int*>(p + 16);
-    if (r.var.exec == PV_EXEC_MULTI_PASS) {
+    if (multi && r.generic) {
       r.proj.tile_count = reinterpret_cast<int64_t*>(p + 32);
       r.proj.tile_offset = r.proj.tile_count + r.proj.n_tiles;
+    } else if (multi) {
+      r.proj.mark_super = reinterpret_cast<unsigned long long*>(p + 32);
+      r.proj.mark_count = reinterpret_cast<unsigned int*>(p + 32 + mark_super_bytes(k.n_rows));
+      r.proj.bits = reinterpret_cast<uint32_t*>(p + 32 + mark_count_bytes(k.n_rows));
     }
     return PV_OK;
   }

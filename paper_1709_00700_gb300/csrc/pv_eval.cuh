@@ -605,9 +605,9 @@ __device__ __forceinline__ void compact_first_eval(Item<SH>& it, const KParams& 
 // by stage for all K rows (a first-stage probe again only when its payload is
 // read), then the loads of the columns the sink reads.  ok[k] is false when a
 // probe missed.
-template <class SH, int K, int NF>
+template <class SH, int K, int NF, class R>
 __device__ __forceinline__ void compact_load_rows(Item<SH> (&it)[K], bool (&ok)[K], const KParams& kp,
-                                                  const uint32_t (&row)[K], const bool (&has)[K]) {
+                                                  const R (&row)[K], const bool (&has)[K]) {
   using JP = typename SH::Probes;
 #pragma unroll
   for (int k = 0; k < K; ++k) {

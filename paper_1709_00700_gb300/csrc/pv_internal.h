@@ -83,10 +83,33 @@ struct ProjOut {
   unsigned long long* cursor;   // single pass: write cursor (zero between runs)
   int64_t* count;               // rows written (min(total, capacity))
   unsigned int* done;           // single pass: block ticket
-  int64_t* tile_count;          // multi pass: matches per tile
-  int64_t* tile_offset;         // multi pass: exclusive prefix of tile_count
+  int64_t* tile_count;          // multi pass, generic kernels: matches per tile (allocation-free entry
+                                // point: tile words, the word before them is the ticket)
+  int64_t* tile_offset;         // multi pass, generic kernels: exclusive prefix of tile_count
   int64_t n_tiles;
+  // multi pass, compiled shapes: matches per kMarkSuper tiles (the counts of the tiles follow), one bit
+  // per row, matches per tile of kMarkTileRows rows
+  unsigned long long* mark_super;
+  unsigned int* mark_count;
+  uint32_t* bits;
 };
+
+// Scratch of the ordered projection: a tile is what one CTA of 256 threads
+// writes out, one bitmap word a thread.
+constexpr int kMarkTileRows = 8192;
+constexpr int kMarkSuper = 64;
+__host__ __device__ inline int64_t mark_tiles(int64_t n_rows) {
+  return n_rows > kMarkTileRows ? (n_rows + kMarkTileRows - 1) / kMarkTileRows : 1;
+}
+inline size_t mark_super_bytes(int64_t n_rows) {
+  return static_cast<size_t>((mark_tiles(n_rows) + kMarkSuper - 1) / kMarkSuper) * 8;
+}
+inline size_t mark_count_bytes(int64_t n_rows) {  // supers and tiles, a multiple of 8
+  return mark_super_bytes(n_rows) + ((static_cast<size_t>(mark_tiles(n_rows)) * 4 + 7) & ~size_t(7));
+}
+inline size_t mark_bytes(int64_t n_rows) {
+  return mark_count_bytes(n_rows) + static_cast<size_t>(mark_tiles(n_rows)) * (kMarkTileRows / 8);
+}
 
 // Grouped aggregation description shared by the group kernels and the host.
 struct GroupDesc {
