@@ -794,6 +794,12 @@ __device__ __forceinline__ void extract_replicated(const GroupDesc& gd, const Gr
 }
 
 
+}  // namespace pv
+
+#include "k_part.cuh"
+
+namespace pv {
+
 // ---------------------------------------------------------------------------
 // Kernels
 // ---------------------------------------------------------------------------
@@ -822,6 +828,7 @@ template <class SH, class Sink, bool PRED> struct GroupRegs {
 template <class SH, bool PRED, bool CHUNK, int U, class Sink>
 __global__ void __maxnreg__((GroupRegs<SH, Sink, PRED>::value)) k_group(const __grid_constant__ KParams kp, const __grid_constant__ GroupDesc gd, const __grid_constant__ GroupOut g) {
   extern __shared__ unsigned long long smem[];
+  if (g.guard != nullptr && __ldcg(g.guard) == 0u) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) *g.out_count = 0;  // extraction runs after this kernel
   Sink sink(gd, g, kp.err, smem);
   sink.init();
@@ -1116,8 +1123,20 @@ static pv_status run_keys(const LaunchCfg& c, const KParams& kp, const GroupDesc
 // extraction kernel.
 template <class SH, int UMASK>
 static pv_status launch_group(const LaunchCfg& c, const KParams& kp, const GroupDesc& gd, const GroupOut& g0,
-                              const pv_variant& v) {
+                              const PartOut& po, const pv_variant& v) {
   GroupOut g = g0;
+  if (po.key != nullptr) {
+    if constexpr (part_hash_ok<SH>()) {
+      if (g.ht == PV_HT_LINEAR) {
+        const pv_status s = run_part<SH, true>(c, kp, gd, g, po);
+        if (s != PV_OK) return s;
+        g.guard = po.ctl + kPartCtlFull;  // the general kernels below run when a range was full
+      }
+    }
+    if constexpr (part_perfect_ok<SH>()) {
+      if (g.ht == PV_HT_PERFECT) return run_part<SH, false>(c, kp, gd, g, po);
+    }
+  }
   const bool multi = v.exec == PV_EXEC_MULTI_PASS;
   const bool local = v.agg == PV_AGG_LOCAL;
   if (multi && (c.compact || c.staged)) return PV_ERR_UNSUPPORTED;  // the key pass has neither form
@@ -1204,6 +1223,8 @@ static void reg_grouped() {
   e.sig = SH::signature();
   e.mode = MODE_GROUPED;
   e.grouped = launch_group<SH, UMASK>;
+  e.part_words = part_perfect_ok<SH>() ? part_words<typename SH::Aggs>() : -1;
+  e.part_hash = part_hash_ok<SH>();
   register_shape(e);
 }
 

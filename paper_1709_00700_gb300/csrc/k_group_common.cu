@@ -22,6 +22,7 @@ __global__ void k_cuckoo_dedupe(const __grid_constant__ GroupOut g) {
 
 __global__ void k_extract(const __grid_constant__ GroupDesc gd, const __grid_constant__ GroupOut g) {
   pdl_wait();  // launched early behind the aggregation kernel
+  if (g.guard != nullptr && __ldcg(g.guard) == 0u) return;
   const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
   if (g.replicas > 1) extract_replicated(gd, g, t, T);

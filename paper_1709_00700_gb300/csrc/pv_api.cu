@@ -115,6 +115,7 @@ struct Result {
   ProjOut proj{};
   GroupDesc gd{};
   GroupOut grp{};
+  PartOut part{};
   int n_cols = 0;
   int col_type[PV_MAX_KEYS + PV_MAX_AGGS]{};
   int64_t rows_cached = -1;
@@ -611,6 +612,63 @@ static pv_status column_stats(pv_ctx* c, pv_col h, int64_t* mn, int64_t* mx) {
 }
 
 
+// Scratch for the partitioned aggregation (k_part.cuh) of a result whose table
+// is global and too large to be updated in place cheaply; without it (not the
+// variant, too few rows, no memory) the general kernels run.
+static void alloc_part(pv_ctx* c, Result& r) {
+  const Canon& k = r.canon;
+  const GroupOut& g = r.grp;
+  const pv_variant& v = r.var;
+  if (r.generic || !r.entry || r.entry->part_words < 0 || v.agg != PV_AGG_GLOBAL || v.exec != PV_EXEC_SINGLE_PASS ||
+      v.threads_per_table == 1 || v.pred == PV_COMPACTED || v.access == PV_STAGED)
+    return;
+  const bool hash = g.ht == PV_HT_LINEAR;
+  if (hash ? !r.entry->part_hash : g.ht != PV_HT_PERFECT) return;
+  const int words = r.entry->part_words;
+  // Where the partitioned kernels are the faster ones (us, general kernels against partitioned): atomics on
+  // tables past 16 MB (1.1M rows, 1e6 groups 43 / 34; 4M rows, 1e7 groups 395 / 112); many rows (20M rows, 1e4
+  // groups 284 / 205; hash table of 3e4 groups 568 / 397); skew, which a perfect array's variant states with
+  // warp_agg (1.1M rows, 1e5 groups 140 / 33).  A small table with fewer rows stays with the general
+  // kernels (4M rows, 1e5 groups 49 / 76).
+  const bool big = g.cap * (g.stride + (hash ? 1 : 0)) * 8 >= (int64_t(16) << 20);
+  const bool many = k.n_rows >= (hash ? int64_t(4) << 20 : int64_t(16) << 20);
+  if (k.n_rows < kPartMinRows || k.n_rows > (int64_t(1) << 31) || (!hash && g.cap < kPartMinSlots) ||
+      !(big || many || (!hash && v.warp_agg)))
+    return;
+  // about 600 ranges of a perfect array (fewer leave SMs idle, more shorten the runs the scatter writes: 60M
+  // rows in 391 ranges 334 us, in 1221 498 us), about 1024 of a hash table (smaller ranges spread hot keys),
+  // of at least 256 slots, at most what an SM's shared memory holds
+  const int max_shift = hash ? 12 : words <= 1 ? 14 : 13;
+  int shift = 8;
+  while (shift < max_shift && (g.cap >> shift) > (hash ? 1024 : 640)) ++shift;
+  if (hash) shift = std::min(shift, g.log2cap);
+  const int64_t parts = (g.cap + (int64_t(1) << shift) - 1) >> shift;
+  if (parts > kPartMaxRanges) return;
+  PartOut po{};
+  po.n_parts = static_cast<int>(parts);
+  po.shift = shift;
+  // a few units per CTA, of rows enough to pay for emptying and reading out a table; evenly filled ranges
+  // whose slots are many next to their rows stay whole, as adding them up again would cost more
+  int64_t unit = std::max<int64_t>({2048, int64_t(2) << shift, k.n_rows / (c->sm_count * 6)});
+  if (!hash && unit < (int64_t(16) << shift) && parts >= c->sm_count) unit = std::max(unit, k.n_rows / parts * 3 / 2);
+  po.unit_rows = static_cast<uint32_t>(unit);
+  const size_t n = (static_cast<size_t>(k.n_rows) + 3) & ~size_t(3);
+  const size_t ctl = 4 * static_cast<size_t>(parts) + 2 + kPartCtlWords + kPartMaxRanges;
+  char* p = static_cast<char*>(dalloc(c, n * (8 * words + 4) + ctl * 4));
+  if (!p) return;
+  r.mem.push_back(p);
+  for (int w = 0; w < words; ++w, p += n * 8) po.val[w] = reinterpret_cast<unsigned long long*>(p);
+  po.key = reinterpret_cast<uint32_t*>(p);
+  po.hist = po.key + n;
+  po.done = po.hist + parts;
+  po.ctl = po.done + parts;
+  po.clear_bytes = (2 * static_cast<size_t>(parts) + kPartCtlWords) * 4;
+  po.off = po.ctl + kPartCtlWords;
+  po.unit_off = po.off + parts + 1;
+  po.cursor = po.unit_off + parts + 1;
+  r.part = po;
+}
+
 static pv_status alloc_result(pv_ctx* c, Result& r) {
   const Canon& k = r.canon;
   auto grab = [&](size_t bytes) -> void* {
@@ -754,6 +812,7 @@ static pv_status alloc_result(pv_ctx* c, Result& r) {
   PV_CUDA(c, cudaMemsetAsync(g.out_count, 0, 16, c->stream));
   r.n_cols = ncol;
   for (int i = 0; i < ncol; ++i) r.col_type[i] = PV_I64;
+  alloc_part(c, r);
   return PV_OK;
 }
 
@@ -776,7 +835,7 @@ static pv_status launch_result(pv_ctx* c, Result& r) {
   } else {
     if (k.mode == MODE_AGGREGATE) s = r.entry->aggregate(L, k.kp, r.agg);
     else if (k.mode == MODE_PROJECT) s = r.entry->project(L, k.kp, r.proj, r.var.exec);
-    else s = r.entry->grouped(L, k.kp, r.gd, r.grp, r.var);
+    else s = r.entry->grouped(L, k.kp, r.gd, r.grp, r.part, r.var);
   }
   if (s == PV_ERR_UNSUPPORTED) return fail(c, s, "no instantiation of this shape for the variant");
   if (s != PV_OK) return fail(c, s, "kernel launch failed");

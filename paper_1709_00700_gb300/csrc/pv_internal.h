@@ -166,6 +166,31 @@ struct GroupOut {
   int64_t* out;
   int64_t out_cap;
   unsigned long long* out_count;
+  // Kernels of a fallback run only when this device word is not 0 (null: always).
+  const uint32_t* guard;
+};
+
+// Scratch of the partitioned grouped aggregation (k_part.cuh), owned by a
+// result; key == nullptr: the result has none.  The words that start at zero
+// (clear_bytes from hist): rows per range, finished units per range, control.
+constexpr int kPartWords = 2;  // value words of a record at most
+enum { kPartCtlUnit = 0, kPartCtlDone = 1, kPartCtlFull = 2, kPartCtlWords = 4 };
+constexpr int kPartMaxRanges = 2048;
+constexpr int64_t kPartMinRows = 1 << 20;   // fewer rows: the general kernels
+constexpr int64_t kPartMinSlots = 1 << 12;  // of a perfect array
+struct PartOut {
+  uint32_t* key;                        // records, by range: group key or slot
+  unsigned long long* val[kPartWords];  //   and aggregate codes
+  uint32_t* hist;                       // [n_parts] rows
+  uint32_t* done;                       // [n_parts] units that added into the global table
+  uint32_t* ctl;                        // next unit, finished CTAs of the count, a range was full
+  uint32_t* off;                        // [n_parts + 1] first record of a range
+  uint32_t* unit_off;                   // [n_parts + 1] first unit of a range
+  uint32_t* cursor;                     // [n_parts, padded to kPartMaxRanges] next record to write
+  size_t clear_bytes;
+  int n_parts;
+  int shift;                            // log2 of the slots of a range
+  uint32_t unit_rows;
 };
 
 // A pipeline program as data, for the generic (interpreted) kernels of
@@ -212,8 +237,12 @@ struct ShapeEntry {
   // Launchers return PV_OK or PV_ERR_UNSUPPORTED (no instantiation for the variant).
   pv_status (*aggregate)(const LaunchCfg&, const KParams&, const AggOut&);
   pv_status (*project)(const LaunchCfg&, const KParams&, const ProjOut&, int exec);
-  pv_status (*grouped)(const LaunchCfg&, const KParams&, const GroupDesc&, const GroupOut&,
+  pv_status (*grouped)(const LaunchCfg&, const KParams&, const GroupDesc&, const GroupOut&, const PartOut&,
                        const pv_variant&);
+  // grouped: value words of a partitioned record (-1: the shape has no
+  // partitioned kernels), and whether its hash tables have them too
+  int part_words;
+  bool part_hash;
 };
 
 void register_shape(const ShapeEntry& e);
