@@ -43,6 +43,7 @@ struct BuildTable {
   void* mem = nullptr;
   size_t slot_bytes = 0;  // bytes of the slot array (rebuilds clear them)
   BuildParams bp{};       // the build pipeline, kept for rebuilds
+  bool built = false;     // payload statistics and the form probes read are known
 };
 
 struct BuildEnv {
@@ -61,7 +62,7 @@ pv_status build_table(const BuildEnv& env, const BuildInput& in, const pv_ht_var
                       int64_t kmax, BuildTable& out, std::string& msg);
 
 // Enqueues the build pipeline of an existing table again (clear, insert,
-// duplicate check): no allocation, no synchronisation; the payload
+// duplicate check; a perfect array's slots only when probes read them): no allocation, no synchronisation; the payload
 // statistics of the first build are kept.
 pv_status rebuild_table(const BuildEnv& env, const BuildTable& t);
 
