@@ -174,12 +174,87 @@ __device__ __forceinline__ uint64_t block_excl_scan(uint64_t v, uint64_t* total)
   return ex;
 }
 
-// Single pass: every warp reserves its matches with one atomicAdd on the
-// output cursor (ballot-free: counts are scanned with shuffles), then each
-// lane writes its rows.  Output order is arbitrary across warps.
+// Bytes of one projected row before projected column C (source column types;
+// payloads are int32); proj_offset<SH, N> is the whole row.
+template <class SH, int C>
+constexpr int proj_offset() {
+  if constexpr (C == 0) {
+    return 0;
+  } else {
+    constexpr int S = SH::Proj::slot_of[C - 1];
+    constexpr int sz = S >= 0 ? static_cast<int>(sizeof(typename At<(S >= 0 ? S : 0), typename SH::Cols::L>::type::T)) : 4;
+    return proj_offset<SH, C - 1>() + sz;
+  }
+}
+
+// A warp's output stage in shared memory, R rows: column C at R * offset(C).
+template <class SH, int R>
+__host__ __device__ constexpr size_t out_stage_bytes() {
+  return (static_cast<size_t>(R) * proj_offset<SH, SH::Proj::N>() + 15) & ~size_t(15);
+}
+
+// Row r of an item into row `slot` of the stage.
+template <class SH, int R>
+__device__ __forceinline__ void stage_out_row(char* st, int slot, Item<SH>& it, int r) {
+  using PJ = typename SH::Proj;
+  static_for<PJ::N>([&](auto c) {
+    constexpr int C = decltype(c)::value;
+    constexpr int S = PJ::slot_of[C];
+    char* col = st + R * proj_offset<SH, C>();
+    if constexpr (S >= 0) {
+      using T = typename At<S, typename SH::Cols::L>::type::T;
+      reinterpret_cast<T*>(col)[slot] = VGet<S>::get(it.v)[r];
+    } else {
+      reinterpret_cast<int32_t*>(col)[slot] = it.pay[-S - 1][r];
+    }
+  });
+}
+
+// The warp's n staged rows to the output at positions reserved with one
+// atomicAdd; rows past the capacity are dropped (overflow).  All lanes.
+template <class SH, int R>
+__device__ __forceinline__ void flush_out_rows(const char* st, int n, const ProjOut& out, bool& overflow) {
+  using PJ = typename SH::Proj;
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  unsigned long long base = 0;
+  if (lane == 0) base = atomicAdd(out.cursor, static_cast<unsigned long long>(n));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  for (int i = lane; i < n; i += 32) {
+    const int64_t pos = static_cast<int64_t>(base) + i;
+    if (pos >= out.capacity) {
+      overflow = true;
+      continue;
+    }
+    static_for<PJ::N>([&](auto c) {
+      constexpr int C = decltype(c)::value;
+      constexpr int S = PJ::slot_of[C];
+      const char* col = st + R * proj_offset<SH, C>();
+      if constexpr (S >= 0) {
+        using T = typename At<S, typename SH::Cols::L>::type::T;
+        static_cast<T*>(out.col[C])[pos] = reinterpret_cast<const T*>(col)[i];
+      } else {
+        static_cast<int32_t*>(out.col[C])[pos] = reinterpret_cast<const int32_t*>(col)[i];
+      }
+    });
+  }
+  __syncwarp();
+}
+
+// Single pass: a warp's matches of a trip (counts are scanned with shuffles)
+// are written at positions reserved with one atomicAdd on the output cursor.
+// The cursor takes about one atomic a nanosecond, so a trip of fewer than
+// kSpFlush rows is staged in shared memory until that many are there: 15M
+// rows with 9% matching, 12 rows a trip, were bound by the cursor (118 us).
+// Output order is arbitrary across warps.
+constexpr int kSpFlush = 64;
+constexpr int kSpStage = 2 * kSpFlush;  // rows staged at most: kSpFlush - 1 and one trip's
 template <class SH, bool PRED, bool CHUNK, int U>
 __global__ void __maxnreg__(128) k_project_sp(const __grid_constant__ KParams kp, const __grid_constant__ ProjOut out) {
+  extern __shared__ float4 spmem[];
+  char* st = reinterpret_cast<char*>(spmem) + (threadIdx.x >> 5) * out_stage_bytes<SH, kSpStage>();
   bool overflow = false;
+  int staged = 0;  // warp-uniform
   for_items_uniform<CHUNK, U>(kp.n_items, [&](const int64_t (&idx)[U]) {
     Item<SH> it[U];
     eval_items<SH, PRED, U>(it, kp, idx);
@@ -189,6 +264,20 @@ __global__ void __maxnreg__(128) k_project_sp(const __grid_constant__ KParams kp
     const int incl = warp_incl_scan(cnt);
     const int total = __shfl_sync(0xffffffffu, incl, 31);
     if (total == 0) return;
+    if (total < kSpFlush) {
+      int slot = staged + incl - cnt;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if ((it[u].mask >> r) & 1u) stage_out_row<SH, kSpStage>(st, slot++, it[u], r);
+      staged += total;
+      if (staged >= kSpFlush) {
+        flush_out_rows<SH, kSpStage>(st, staged, out, overflow);
+        staged = 0;
+      }
+      return;
+    }
     unsigned long long base = 0;
     if ((threadIdx.x & 31) == 31) base = atomicAdd(out.cursor, static_cast<unsigned long long>(total));
     base = __shfl_sync(0xffffffffu, base, 31);
@@ -205,6 +294,7 @@ __global__ void __maxnreg__(128) k_project_sp(const __grid_constant__ KParams kp
       }
     }
   });
+  if (staged > 0) flush_out_rows<SH, kSpStage>(st, staged, out, overflow);
   if (overflow) set_error(kp.err, PV_ERR_OUTPUT_OVERFLOW);
   __shared__ bool last;
   __syncthreads();
@@ -538,75 +628,10 @@ __global__ void __maxnreg__(128) k_aggregate_compact(const __grid_constant__ KPa
   aggregate_epilogue<SH>(acc, out);
 }
 
-// Bytes of one projected row before projected column C (source column types;
-// payloads are int32); proj_offset<SH, N> is the whole row.
-template <class SH, int C>
-constexpr int proj_offset() {
-  if constexpr (C == 0) {
-    return 0;
-  } else {
-    constexpr int S = SH::Proj::slot_of[C - 1];
-    constexpr int sz = S >= 0 ? static_cast<int>(sizeof(typename At<(S >= 0 ? S : 0), typename SH::Cols::L>::type::T)) : 4;
-    return proj_offset<SH, C - 1>() + sz;
-  }
-}
-
 // Output rows a warp stages in shared memory before it reserves their
 // positions: a flush starts at 64 rows, and one drain adds at most 32 * K.
 template <int K>
 __host__ __device__ constexpr int out_stage_rows() { return 32 * (2 + K); }
-template <class SH, int K>
-__host__ __device__ constexpr size_t out_stage_bytes() {
-  return (static_cast<size_t>(out_stage_rows<K>()) * proj_offset<SH, SH::Proj::N>() + 15) & ~size_t(15);
-}
-
-// Row `slot` of a warp's output stage (column C at stage + rows * offset(C)).
-template <class SH, int K>
-__device__ __forceinline__ void stage_out_row(char* st, int slot, Item<SH>& it) {
-  using PJ = typename SH::Proj;
-  static_for<PJ::N>([&](auto c) {
-    constexpr int C = decltype(c)::value;
-    constexpr int S = PJ::slot_of[C];
-    char* col = st + out_stage_rows<K>() * proj_offset<SH, C>();
-    if constexpr (S >= 0) {
-      using T = typename At<S, typename SH::Cols::L>::type::T;
-      reinterpret_cast<T*>(col)[slot] = VGet<S>::get(it.v)[0];
-    } else {
-      reinterpret_cast<int32_t*>(col)[slot] = it.pay[-S - 1][0];
-    }
-  });
-}
-
-// The warp's n staged rows to the output at positions reserved with one
-// atomicAdd; rows past the capacity are dropped (overflow).  All lanes.
-template <class SH, int K>
-__device__ __forceinline__ void flush_out_rows(const char* st, int n, const ProjOut& out, bool& overflow) {
-  using PJ = typename SH::Proj;
-  const int lane = threadIdx.x & 31;
-  __syncwarp();
-  unsigned long long base = 0;
-  if (lane == 0) base = atomicAdd(out.cursor, static_cast<unsigned long long>(n));
-  base = __shfl_sync(0xffffffffu, base, 0);
-  for (int i = lane; i < n; i += 32) {
-    const int64_t pos = static_cast<int64_t>(base) + i;
-    if (pos >= out.capacity) {
-      overflow = true;
-      continue;
-    }
-    static_for<PJ::N>([&](auto c) {
-      constexpr int C = decltype(c)::value;
-      constexpr int S = PJ::slot_of[C];
-      const char* col = st + out_stage_rows<K>() * proj_offset<SH, C>();
-      if constexpr (S >= 0) {
-        using T = typename At<S, typename SH::Cols::L>::type::T;
-        static_cast<T*>(out.col[C])[pos] = reinterpret_cast<const T*>(col)[i];
-      } else {
-        static_cast<int32_t*>(out.col[C])[pos] = reinterpret_cast<const int32_t*>(col)[i];
-      }
-    });
-  }
-  __syncwarp();
-}
 
 // Compacted single-pass PROJECT: the rows that survive the first operation
 // are queued per warp; at each drain every lane takes its queued rows through
@@ -624,7 +649,7 @@ __global__ void __maxnreg__(48) k_project_compact(const __grid_constant__ KParam
                                                    const __grid_constant__ ProjOut out) {
   extern __shared__ uint32_t qmem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  char* ost = reinterpret_cast<char*>(qmem + nwarps * queue_cap<K>()) + warp * out_stage_bytes<SH, K>();
+  char* ost = reinterpret_cast<char*>(qmem + nwarps * queue_cap<K>()) + warp * out_stage_bytes<SH, out_stage_rows<K>()>();
   bool overflow = false;
   int staged = 0;  // warp-uniform
   for_rows_compacted<SH, K, 1, true, FI>(kp, qmem + warp * queue_cap<K>(),
@@ -635,15 +660,15 @@ __global__ void __maxnreg__(48) k_project_compact(const __grid_constant__ KParam
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const unsigned b = __ballot_sync(0xffffffffu, ok[k]);
-      if (ok[k]) stage_out_row<SH, K>(ost, staged + __popc(b & ((1u << lane) - 1u)), it[k]);
+      if (ok[k]) stage_out_row<SH, out_stage_rows<K>()>(ost, staged + __popc(b & ((1u << lane) - 1u)), it[k], 0);
       staged += __popc(b);
     }
     if (staged >= 64) {
-      flush_out_rows<SH, K>(ost, staged, out, overflow);
+      flush_out_rows<SH, out_stage_rows<K>()>(ost, staged, out, overflow);
       staged = 0;
     }
   });
-  if (staged > 0) flush_out_rows<SH, K>(ost, staged, out, overflow);
+  if (staged > 0) flush_out_rows<SH, out_stage_rows<K>()>(ost, staged, out, overflow);
   if (overflow) set_error(kp.err, PV_ERR_OUTPUT_OVERFLOW);
   __shared__ bool last;
   __syncthreads();
@@ -663,7 +688,7 @@ __global__ void __maxnreg__(48) k_project_compact(const __grid_constant__ KParam
 template <class SH, int K>
 static pv_status launch_proj_compact_k(const LaunchCfg& c, const KParams& kp, const ProjOut& out) {
   auto k = c.first_items == 2 ? k_project_compact<SH, K, first_items_max<SH>()> : k_project_compact<SH, K, 1>;
-  const size_t smem = static_cast<size_t>(c.block / 32) * (queue_cap<K>() * 4 + out_stage_bytes<SH, K>());
+  const size_t smem = static_cast<size_t>(c.block / 32) * (queue_cap<K>() * 4 + out_stage_bytes<SH, out_stage_rows<K>()>());
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
     return PV_ERR_UNSUPPORTED;
@@ -740,10 +765,14 @@ template <class SH, bool P, bool C, int U>
 static pv_status launch_proj_t(const LaunchCfg& c, const KParams& kp, const ProjOut& out, int exec) {
   if (exec == PV_EXEC_SINGLE_PASS) {
     auto k = k_project_sp<SH, P, C, U>;
-    const int grid = grid_for(c, reinterpret_cast<const void*>(k), 0, kp.n_items, static_cast<int64_t>(c.block) * U);
+    const size_t smem = static_cast<size_t>(c.block / 32) * out_stage_bytes<SH, kSpStage>();
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+      return PV_ERR_UNSUPPORTED;
+    const int grid = grid_for(c, reinterpret_cast<const void*>(k), smem, kp.n_items, static_cast<int64_t>(c.block) * U);
     if (grid <= 0) return PV_ERR_UNSUPPORTED;
     kmark(c);
-    k<<<grid, c.block, 0, c.stream>>>(kp, out);
+    k<<<grid, c.block, smem, c.stream>>>(kp, out);
     kmark(c);
     ++*c.launches;
   } else {
