@@ -860,6 +860,19 @@ __global__ void __maxnreg__((GroupRegs<SH, Sink, PRED>::value)) k_group(const __
       eval_items<SH, PRED, U>(it, kp, idx);
       consume(it);
     });
+  } else if constexpr (!CHUNK && first_slot<SH>() >= 0) {
+    if (kp.prefetch == 0) {
+      for_items_ahead<SH, U>(kp, [&](Item<SH> (&it)[U], const int64_t (&idx)[U]) {
+        eval_items<SH, false, U, true>(it, kp, idx);
+        consume(it);
+      });
+    } else {
+      for_items_pf<SH, CHUNK, U, first_stage_slots<SH>()>(kp, [&](const int64_t (&idx)[U]) {
+        Item<SH> it[U];
+        eval_items<SH, PRED, U>(it, kp, idx);
+        consume(it);
+      });
+    }
   } else {
     for_items_pf<SH, CHUNK, U, first_stage_slots<SH>()>(kp, [&](const int64_t (&idx)[U]) {
       Item<SH> it[U];

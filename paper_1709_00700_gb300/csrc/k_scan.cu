@@ -249,15 +249,14 @@ __device__ __forceinline__ void flush_out_rows(const char* st, int n, const Proj
 // Output order is arbitrary across warps.
 constexpr int kSpFlush = 64;
 constexpr int kSpStage = 2 * kSpFlush;  // rows staged at most: kSpFlush - 1 and one trip's
+// At most 64 registers up to two items, so that blocks of 1024 threads launch.
 template <class SH, bool PRED, bool CHUNK, int U>
-__global__ void __maxnreg__(128) k_project_sp(const __grid_constant__ KParams kp, const __grid_constant__ ProjOut out) {
+__global__ void __maxnreg__((U <= 2 ? 64 : 128)) k_project_sp(const __grid_constant__ KParams kp, const __grid_constant__ ProjOut out) {
   extern __shared__ float4 spmem[];
   char* st = reinterpret_cast<char*>(spmem) + (threadIdx.x >> 5) * out_stage_bytes<SH, kSpStage>();
   bool overflow = false;
   int staged = 0;  // warp-uniform
-  for_items_uniform<CHUNK, U>(kp.n_items, [&](const int64_t (&idx)[U]) {
-    Item<SH> it[U];
-    eval_items<SH, PRED, U>(it, kp, idx);
+  auto write_items = [&](Item<SH> (&it)[U]) {
     int cnt = 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) cnt += __popc(it[u].mask);
@@ -293,7 +292,19 @@ __global__ void __maxnreg__(128) k_project_sp(const __grid_constant__ KParams kp
         }
       }
     }
-  });
+  };
+  if constexpr (!PRED && !CHUNK && first_slot<SH>() >= 0) {
+    for_items_ahead<SH, U>(kp, [&](Item<SH> (&it)[U], const int64_t (&idx)[U]) {
+      eval_items<SH, false, U, true>(it, kp, idx);
+      write_items(it);
+    });
+  } else {
+    for_items_uniform<CHUNK, U>(kp.n_items, [&](const int64_t (&idx)[U]) {
+      Item<SH> it[U];
+      eval_items<SH, PRED, U>(it, kp, idx);
+      write_items(it);
+    });
+  }
   if (staged > 0) flush_out_rows<SH, kSpStage>(st, staged, out, overflow);
   if (overflow) set_error(kp.err, PV_ERR_OUTPUT_OVERFLOW);
   __shared__ bool last;

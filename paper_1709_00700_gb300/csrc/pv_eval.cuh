@@ -8,9 +8,18 @@
 
 namespace pv {
 
+// Slot of the column a branched pipeline reads first (-1: no filter, no probe).
+template <class SH>
+constexpr int first_slot() {
+  if constexpr (SH::Where::N > 0) return At<0, typename SH::Where::L>::type::slot;
+  else if constexpr (SH::Probes::N > 0) return SH::Probes::slot_of[0];
+  else return -1;
+}
+
 // Evaluates U items stage by stage so that the loads of all U items of one
-// stage are in flight together (loop unrolling, Section 6).
-template <class SH, bool PRED, int U>
+// stage are in flight together (loop unrolling, Section 6).  FIRST (branched):
+// the items already hold the column of first_slot().
+template <class SH, bool PRED, int U, bool FIRST = false>
 __device__ __forceinline__ void eval_items(Item<SH> (&it)[U], const KParams& kp, const int64_t (&idx)[U]) {
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -27,7 +36,7 @@ __device__ __forceinline__ void eval_items(Item<SH> (&it)[U], const KParams& kp,
     for (int u = 0; u < U; ++u)
       static_for<W::N>([&](auto j) { it[u].mask &= pred_bits<SH, decltype(j)::value>(it[u], kp); });
   } else {
-    uint32_t loaded = 0;
+    uint32_t loaded = FIRST && W::N > 0 ? 1u << (first_slot<SH>() & 31) : 0u;
     static_for<W::N>([&](auto j) {
       constexpr int J = decltype(j)::value;
       constexpr int S = At<J, typename W::L>::type::slot;
@@ -44,7 +53,7 @@ __device__ __forceinline__ void eval_items(Item<SH> (&it)[U], const KParams& kp,
   static_for<JP::N>([&](auto j) {
     constexpr int J = decltype(j)::value;
     constexpr int S = JP::slot_of[J];
-    if constexpr (!PRED && !((W::slots >> S) & 1u)) {
+    if constexpr (!PRED && !((W::slots >> S) & 1u) && !(FIRST && J == 0 && W::N == 0)) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
         if (it[u].mask) load_slots<SH, (1u << S)>(it[u], kp, idx[u]);
@@ -192,6 +201,44 @@ __device__ __forceinline__ void for_items_pf(const KParams& kp, F&& f) {
 #pragma unroll
     for (int u = 0; u < U; ++u) idx[u] = base + u * T;
     f(idx);
+  }
+}
+
+// Branched grid-stride item loop (trips and items of for_items) that loads the
+// first column of a warp's next trip before it evaluates this one: the first
+// read of every trip is whole columns at DRAM latency, and the reads behind it
+// depend on it (Q5-shaped chain 428 -> 416 us; in the compacted loop the
+// registers it holds cost more than it gives, 163 -> 181 us for the star join).  f(items, idx) evaluates with FIRST.  All lanes of a warp run
+// every trip, items past the end empty.
+template <class SH, int U, class F>
+__device__ __forceinline__ void for_items_ahead(const KParams& kp, F&& f) {
+  constexpr int S = first_slot<SH>();
+  static_assert(S >= 0, "the pipeline reads no column before its sink");
+  const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  Item<SH> next[U];
+  auto load_next = [&](int64_t wb) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t item = wb + lane + u * T;
+      const int64_t left = kp.n_rows - item * 4;
+      next[u].nvalid = left >= 4 ? 4 : (left > 0 ? static_cast<int>(left) : 0);
+      load_slots<SH, (1u << S)>(next[u], kp, item);
+    }
+  };
+  load_next(t - lane);
+  for (int64_t wb = t - lane; wb < kp.n_items; wb += U * T) {
+    Item<SH> it[U];
+    int64_t idx[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      idx[u] = wb + lane + u * T;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) VGet<S>::get(it[u].v)[r] = VGet<S>::get(next[u].v)[r];
+    }
+    load_next(wb + U * T);
+    f(it, idx);
   }
 }
 
