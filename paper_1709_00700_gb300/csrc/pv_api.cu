@@ -177,7 +177,10 @@ void* dalloc(pv_ctx* c, size_t bytes) {
   bytes = (bytes + 255) & ~size_t(255);
   if (c->alloc) return c->alloc(bytes, c->user);
   void* p = nullptr;
-  if (cudaMallocAsync(&p, bytes, c->stream) != cudaSuccess) return nullptr;
+  if (cudaMallocAsync(&p, bytes, c->stream) != cudaSuccess) {
+    cudaGetLastError();  // or the next launch check would report this allocation
+    return nullptr;
+  }
   return p;
 }
 
