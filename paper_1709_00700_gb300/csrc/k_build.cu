@@ -331,6 +331,7 @@ __global__ void __launch_bounds__(256) k_build_direct(const __grid_constant__ Bu
     n = d < static_cast<unsigned long long>(n) ? static_cast<int64_t>(d) : n;
   }
   const int64_t T = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int lane = threadIdx.x & 31;
   for (int64_t r0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; r0 < n; r0 += K * T) {
     bool pass[K];
 #pragma unroll
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(256) k_build_direct(const __grid_constant__ Bu
         set_error(bp.err, PV_ERR_KEY_OUT_OF_RANGE);
         continue;
       }
-      uint32_t old, mine;
+      uint32_t mine;
       if constexpr (CODES) {
         const int64_t c = static_cast<int64_t>(static_cast<int32_t>(pay[k])) - h.code_base;
         if (c < 1 || c > 255) {
@@ -364,13 +365,30 @@ __global__ void __launch_bounds__(256) k_build_direct(const __grid_constant__ Bu
         }
         const int sh = 8 * static_cast<int>(slot[k] & 3);
         mine = 0xFFu << sh;
-        old = atomicOr(reinterpret_cast<uint32_t*>(const_cast<uint8_t*>(h.codes)) + (slot[k] >> 2),
-                       static_cast<uint32_t>(c) << sh);
+        const uint32_t old = atomicOr(reinterpret_cast<uint32_t*>(const_cast<uint8_t*>(h.codes)) + (slot[k] >> 2),
+                                      static_cast<uint32_t>(c) << sh);
+        if (old & mine) set_error(bp.err, PV_ERR_DUP_BUILD_KEY);
       } else {
+        // Rows of neighbouring keys meet in one word, where their atomics take turns (3M keys in table order:
+        // 56 us row by row, 40 us through the slots, 22 us so): when many lanes have a row, those of the first
+        // and of the last one's word set their bits with one atomic each.  (Warp-wide votes outside the branch
+        // keep the four rows' loads apart: 15M rows, 30% kept, 141 us against 80.)
+        const uint32_t word = static_cast<uint32_t>(slot[k] >> 5);
+        const unsigned active = __activemask();
+        unsigned lanes = 1u << lane;
         mine = 1u << (slot[k] & 31);
-        old = atomicOr(const_cast<uint32_t*>(h.bits) + (slot[k] >> 5), mine);
+        uint32_t all = mine;
+        if (__popc(active) > 8) {
+          const unsigned first = __ballot_sync(active, word == __shfl_sync(active, word, __ffs(active) - 1));
+          const unsigned last = __ballot_sync(active, word == __shfl_sync(active, word, 31 - __clz(active)));
+          lanes = (first >> lane) & 1u ? first : (last >> lane) & 1u ? last : lanes;
+          if (lanes & (lanes - 1)) all = __reduce_or_sync(lanes, mine);
+        }
+        bool dup = __popc(all) != __popc(lanes);
+        if (lane == __ffs(lanes) - 1)
+          dup = (atomicOr(const_cast<uint32_t*>(h.bits) + (slot[k] >> 5), all) & all) != 0 || dup;
+        if (dup) set_error(bp.err, PV_ERR_DUP_BUILD_KEY);
       }
-      if (old & mine) set_error(bp.err, PV_ERR_DUP_BUILD_KEY);
     }
   }
 }
