@@ -7,6 +7,7 @@
 //     written in table order): matches are marked as bits and counted, then
 //     written; the allocation-free entry point does it in one kernel with a
 //     chained prefix sum.
+#include <algorithm>
 #include <mutex>
 
 #include "pv_eval.cuh"
@@ -361,14 +362,14 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const __grid_constant__ Proj
 // ---------------------------------------------------------------------------
 // Ordered projection.  A first kernel streams the filter columns and leaves one
 // bit per row (n / 8 bytes, which stay in L2) and the matches per tile of 8192
-// rows and per 64 tiles; the second takes a tile per CTA: its first output
-// position is the sum of the counts before it (at most 63 tiles plus one word
-// per 64 tiles, so no scan kernel), its set bits become a row list in shared
-// memory, and the listed rows are read and written one per lane, coalesced.
-// The filter runs once and the projected columns are read for matching rows
-// only: bound by the filter columns' bytes.  Filtering twice around a scan
-// kernel took 97 + 13 + 146 us for 50M rows with 2% matching (the query with
-// its result delivered 264 us, now 122 us).
+// rows and per super of 16 tiles; the second takes a tile, or a part of one, per
+// CTA: its first output position is the sum of the counts before it (supers,
+// tiles of the super, words of the tile, so no scan kernel), its set bits become
+// a row list in shared memory, and the listed rows are read and written one per
+// lane, coalesced.  The filter runs once and the projected columns are read for
+// matching rows only: bound by the filter columns' bytes.  Filtering twice
+// around a scan kernel took 97 + 13 + 146 us for 50M rows with 2% matching (the
+// query with its result delivered 264 us, now 122 us).
 // ---------------------------------------------------------------------------
 // The shape's filters and probes alone (no sink).
 template <class SH>
@@ -404,34 +405,40 @@ __global__ void __maxnreg__(64) k_project_mark(const __grid_constant__ KParams k
     if (lane == 0 && count != 0) {
       const int64_t tile = unit * (128 * U) / kMarkTileRows;
       atomicAdd(out.mark_count + tile, static_cast<unsigned int>(count));
-      atomicAdd(out.mark_super + tile / kMarkSuper, static_cast<unsigned long long>(count));
+      atomicAdd(out.mark_super + (tile >> out.mark_shift), static_cast<unsigned long long>(count));
     }
   }
   pdl_launch_dependents();
 }
 
+// A CTA's unit is a tile's 2^split-th part: few rows are spread over the SMs, as
+// a whole tile is 8 trips of dependent loads per lane.
 template <class SH>
 __global__ void __launch_bounds__(kMarkTileRows / 32) k_project_emit(const __grid_constant__ KParams kp,
-                                                                     const __grid_constant__ ProjOut out) {
-  __shared__ uint16_t list[kMarkTileRows];  // matching rows of the tile, in order
+                                                                     const __grid_constant__ ProjOut out, int split) {
+  __shared__ uint16_t list[kMarkTileRows];  // matching rows of the unit, in order
   pdl_wait();  // launched early behind the mark kernel
+  constexpr int TW = kMarkTileRows / 32;
+  const int uw = TW >> split;  // words of a unit
   const int64_t n_words = (kp.n_rows + 31) >> 5;
-  const int64_t n_tiles = mark_tiles(kp.n_rows);
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t word = tile * (kMarkTileRows / 32) + threadIdx.x;
-    uint32_t w = word < n_words ? out.bits[word] : 0u;
-    uint64_t before = 0;  // matches of earlier tiles, this thread's share
-    const int64_t super = tile / kMarkSuper;
+  const int64_t n_units = n_words > uw ? (n_words + uw - 1) / uw : 1;
+  for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
+    const int64_t word0 = unit * uw, tile = unit >> split;
+    const int64_t word = word0 + threadIdx.x;
+    uint32_t w = threadIdx.x < uw && word < n_words ? out.bits[word] : 0u;
+    uint64_t before = 0;  // matches of earlier units, this thread's share
+    const int64_t super = tile >> out.mark_shift;
     for (int64_t i = threadIdx.x; i < super; i += blockDim.x) before += out.mark_super[i];
-    if (super * kMarkSuper + threadIdx.x < tile) before += out.mark_count[super * kMarkSuper + threadIdx.x];
-    // one scan for both sums: the tile's matches (at most 8192) in the low 16 bits
+    for (int64_t i = (super << out.mark_shift) + threadIdx.x; i < tile; i += blockDim.x) before += out.mark_count[i];
+    if (tile * TW + threadIdx.x < word0) before += __popc(out.bits[tile * TW + threadIdx.x]);
+    // one scan for both sums: the unit's matches (at most 8192) in the low 16 bits
     uint64_t sums;
     int p = static_cast<int>(block_excl_scan((before << 16) | static_cast<uint64_t>(__popc(w)), &sums) & 0xFFFFu);
     const int total = static_cast<int>(sums & 0xFFFFu);
     const int64_t base = static_cast<int64_t>(sums >> 16);
     for (; w != 0; w &= w - 1) list[p++] = static_cast<uint16_t>(threadIdx.x * 32 + __ffs(w) - 1);
     __syncthreads();
-    constexpr int K = 2;  // rows of a lane read together
+    constexpr int K = 4;  // rows of a lane read together
     for (int i = threadIdx.x; i < total; i += K * blockDim.x) {
       Item<SH> it[K];
       bool ok[K], has[K];
@@ -440,7 +447,7 @@ __global__ void __launch_bounds__(kMarkTileRows / 32) k_project_emit(const __gri
       for (int k = 0; k < K; ++k) {
         const int j = i + k * blockDim.x;
         has[k] = j < total;
-        rows[k] = tile * kMarkTileRows + (has[k] ? list[j] : 0);
+        rows[k] = word0 * 32 + (has[k] ? list[j] : 0);
       }
       compact_load_rows<SH, K, 1>(it, ok, kp, rows, has);
 #pragma unroll
@@ -449,12 +456,26 @@ __global__ void __launch_bounds__(kMarkTileRows / 32) k_project_emit(const __gri
         if (ok[k] && at < out.capacity) write_row<SH>(out, it[k], 0, at);
       }
     }
-    if (tile == n_tiles - 1 && threadIdx.x == 0) {
+    if (unit == n_units - 1 && threadIdx.x == 0) {
       const int64_t n = base + total;
       *out.count = n < out.capacity ? n : out.capacity;
       if (n > out.capacity) set_error(kp.err, PV_ERR_OUTPUT_OVERFLOW);
     }
     __syncthreads();  // the list is free again
+  }
+  // The last CTA leaves the counters at zero for the next run: a clear ahead of the marks was a launch of its own
+  // (1M rows 12.3 us).
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(out.done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (last) {
+    const int64_t n_tiles = mark_tiles(kp.n_rows);
+    for (int64_t i = threadIdx.x; i < n_tiles; i += blockDim.x) out.mark_count[i] = 0;
+    for (int64_t i = threadIdx.x; i <= (n_tiles - 1) >> out.mark_shift; i += blockDim.x) out.mark_super[i] = 0;
+    if (threadIdx.x == 0) *out.done = 0;
   }
 }
 
@@ -777,44 +798,54 @@ pv_status launch_tile_scan(const LaunchCfg& c, const ProjOut& out, int32_t* err)
 }
 
 template <class SH, bool P, bool C, int U>
-static pv_status launch_proj_t(const LaunchCfg& c, const KParams& kp, const ProjOut& out, int exec) {
-  if (exec == PV_EXEC_SINGLE_PASS) {
-    auto k = k_project_sp<SH, P, C, U, U == 1 ? 64 : 128>;
-    if constexpr (U == 2)
-      if (c.block > 512) k = k_project_sp<SH, P, C, U, 64>;
-    const size_t smem = static_cast<size_t>(c.block / 32) * out_stage_bytes<SH, kSpStage>();
-    // the kernel's static shared memory counts too: 48 KB of stages (12-byte rows, 1024 threads) need the attribute
-    if (smem >= 40 * 1024 &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
-      return PV_ERR_UNSUPPORTED;
-    const int grid = grid_for(c, reinterpret_cast<const void*>(k), smem, kp.n_items, static_cast<int64_t>(c.block) * U);
-    if (grid <= 0) return PV_ERR_UNSUPPORTED;
-    kmark(c);
-    k<<<grid, c.block, smem, c.stream>>>(kp, out);
-    kmark(c);
-    ++*c.launches;
-  } else {
-    // chunked or coalesced access gives the same rows in the same order: one mapping serves both
-    auto km = k_project_mark<SH, P, U>;
-    auto ke = k_project_emit<SH>;
-    LaunchCfg ce = c;
-    ce.block = kMarkTileRows / 32;
-    ce.grid_mult = 0;
-    const int gm = grid_for(c, reinterpret_cast<const void*>(km), 0, kp.n_items, static_cast<int64_t>(c.block) * U);
-    const int ge = grid_for(ce, reinterpret_cast<const void*>(ke), 0, mark_tiles(kp.n_rows), 1);
-    if (gm <= 0 || ge <= 0) return PV_ERR_UNSUPPORTED;
-    if (cudaMemsetAsync(out.mark_super, 0, mark_count_bytes(kp.n_rows), c.stream) != cudaSuccess) return PV_ERR_CUDA;
-    kmark(c);
-    km<<<gm, c.block, 0, c.stream>>>(kp, out);
-    kmark(c);
-    kmark(c);
-    cudaError_t e = c.mark ? (ke<<<ge, ce.block, 0, c.stream>>>(kp, out), cudaSuccess)
-                           : pdl_launch(ke, dim3(ge), dim3(ce.block), 0, c.stream, kp, out);
-    kmark(c);
-    *c.launches += 2;
-    if (e != cudaSuccess) return PV_ERR_CUDA;
-  }
+static pv_status launch_proj_sp(const LaunchCfg& c, const KParams& kp, const ProjOut& out) {
+  auto k = k_project_sp<SH, P, C, U, U == 1 ? 64 : 128>;
+  if constexpr (U == 2)
+    if (c.block > 512) k = k_project_sp<SH, P, C, U, 64>;
+  const size_t smem = static_cast<size_t>(c.block / 32) * out_stage_bytes<SH, kSpStage>();
+  // the kernel's static shared memory counts too: 48 KB of stages (12-byte rows, 1024 threads) need the attribute
+  if (smem >= 40 * 1024 &&
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    return PV_ERR_UNSUPPORTED;
+  const int grid = grid_for(c, reinterpret_cast<const void*>(k), smem, kp.n_items, static_cast<int64_t>(c.block) * U);
+  if (grid <= 0) return PV_ERR_UNSUPPORTED;
+  kmark(c);
+  k<<<grid, c.block, smem, c.stream>>>(kp, out);
+  kmark(c);
+  ++*c.launches;
   return cudaGetLastError() == cudaSuccess ? PV_OK : PV_ERR_CUDA;
+}
+
+// Ordered projection.  The rows and their order do not depend on access and
+// items_per_thread, so the kernels choose both: the marks take 4 items a lane
+// once that leaves an SM four warps with a unit each (10M rows, one filter,
+// 10% matching: 72 us with one item, 37 with four; 100K rows 6.9 / 8.2).  A
+// tile is split until an SM has three units, at most into 8 (100K rows, all
+// matching: 14 us by whole tiles, 8 by counting twice).
+template <class SH, bool P>
+static pv_status launch_proj_ordered(const LaunchCfg& c, const KParams& kp, const ProjOut& out) {
+  const bool wide = kp.n_items >= static_cast<int64_t>(512) * c.sm_count;
+  auto km = wide ? k_project_mark<SH, P, 4> : k_project_mark<SH, P, 1>;
+  auto ke = k_project_emit<SH>;
+  LaunchCfg ce = c;
+  ce.block = kMarkTileRows / 32;
+  ce.grid_mult = 0;
+  const int gm = grid_for(c, reinterpret_cast<const void*>(km), 0, kp.n_items,
+                          static_cast<int64_t>(c.block) * (wide ? 4 : 1));
+  const int resident = grid_for(ce, reinterpret_cast<const void*>(ke), 0, INT32_MAX, 1);
+  if (gm <= 0 || resident <= 0) return PV_ERR_UNSUPPORTED;
+  int split = 0;
+  while (split < 3 && (mark_tiles(kp.n_rows) << split) < 3 * static_cast<int64_t>(c.sm_count)) ++split;
+  const int ge = static_cast<int>(std::min<int64_t>(resident, mark_tiles(kp.n_rows) << split));
+  kmark(c);
+  km<<<gm, c.block, 0, c.stream>>>(kp, out);
+  kmark(c);
+  kmark(c);
+  cudaError_t e = c.mark ? (ke<<<ge, ce.block, 0, c.stream>>>(kp, out, split), cudaSuccess)
+                         : pdl_launch(ke, dim3(ge), dim3(ce.block), 0, c.stream, kp, out, split);
+  kmark(c);
+  *c.launches += 2;
+  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? PV_OK : PV_ERR_CUDA;
 }
 
 template <class SH>
@@ -833,16 +864,17 @@ static pv_status launch_agg(const LaunchCfg& c, const KParams& kp, const AggOut&
 
 template <class SH>
 static pv_status launch_proj(const LaunchCfg& c, const KParams& kp, const ProjOut& out, int exec) {
-  using F = pv_status (*)(const LaunchCfg&, const KParams&, const ProjOut&, int);
+  using F = pv_status (*)(const LaunchCfg&, const KParams&, const ProjOut&);
   static const F tab[2][2][3] = {
-      {{launch_proj_t<SH, false, false, 1>, launch_proj_t<SH, false, false, 2>, launch_proj_t<SH, false, false, 4>},
-       {launch_proj_t<SH, false, true, 1>, launch_proj_t<SH, false, true, 2>, launch_proj_t<SH, false, true, 4>}},
-      {{launch_proj_t<SH, true, false, 1>, launch_proj_t<SH, true, false, 2>, launch_proj_t<SH, true, false, 4>},
-       {launch_proj_t<SH, true, true, 1>, launch_proj_t<SH, true, true, 2>, launch_proj_t<SH, true, true, 4>}}};
+      {{launch_proj_sp<SH, false, false, 1>, launch_proj_sp<SH, false, false, 2>, launch_proj_sp<SH, false, false, 4>},
+       {launch_proj_sp<SH, false, true, 1>, launch_proj_sp<SH, false, true, 2>, launch_proj_sp<SH, false, true, 4>}},
+      {{launch_proj_sp<SH, true, false, 1>, launch_proj_sp<SH, true, false, 2>, launch_proj_sp<SH, true, false, 4>},
+       {launch_proj_sp<SH, true, true, 1>, launch_proj_sp<SH, true, true, 2>, launch_proj_sp<SH, true, true, 4>}}};
   if (c.compact) return c.compact_probes != 1 ? PV_ERR_UNSUPPORTED : launch_proj_compact<SH>(c, kp, out, exec);
   const int ui = c.U == 1 ? 0 : c.U == 2 ? 1 : c.U == 4 ? 2 : -1;
   if (ui < 0) return PV_ERR_UNSUPPORTED;
-  return tab[c.pred][c.chunk][ui](c, kp, out, exec);
+  if (exec == PV_EXEC_SINGLE_PASS) return tab[c.pred][c.chunk][ui](c, kp, out);
+  return c.pred ? launch_proj_ordered<SH, true>(c, kp, out) : launch_proj_ordered<SH, false>(c, kp, out);
 }
 
 template <class SH>

@@ -708,7 +708,8 @@ static pv_status alloc_result(pv_ctx* c, Result& r) {
     r.proj.n_tiles = std::max<int64_t>(1, (k.kp.n_items + tile_items - 1) / tile_items);
     const bool multi = r.var.exec == PV_EXEC_MULTI_PASS;
     const size_t scratch = !multi ? 0 : r.generic ? 16 * static_cast<size_t>(r.proj.n_tiles) : mark_bytes(k.n_rows);
-    const size_t ctl = 32 + (multi && r.generic ? scratch : 0);  // zeroed here; the marks are cleared by each run
+    // zero between runs; the marks' bits need no clearing
+    const size_t ctl = 32 + (!multi ? 0 : r.generic ? scratch : mark_count_bytes(k.n_rows));
     char* p = static_cast<char*>(grab(32 + scratch));
     if (!p) return fail(c, PV_ERR_OOM, "allocator returned NULL");
     PV_CUDA(c, cudaMemsetAsync(p, 0, ctl, c->stream));
@@ -719,6 +720,7 @@ static pv_status alloc_result(pv_ctx* c, Result& r) {
       r.proj.tile_count = reinterpret_cast<int64_t*>(p + 32);
       r.proj.tile_offset = r.proj.tile_count + r.proj.n_tiles;
     } else if (multi) {
+      r.proj.mark_shift = mark_shift(k.n_rows);
       r.proj.mark_super = reinterpret_cast<unsigned long long*>(p + 32);
       r.proj.mark_count = reinterpret_cast<unsigned int*>(p + 32 + mark_super_bytes(k.n_rows));
       r.proj.bits = reinterpret_cast<uint32_t*>(p + 32 + mark_count_bytes(k.n_rows));
