@@ -245,20 +245,24 @@ __device__ __forceinline__ void flush_out_rows(const char* st, int n, const Proj
 // Single pass: a warp's matches of a trip (counts are scanned with shuffles)
 // are written at positions reserved with one atomicAdd on the output cursor.
 // The cursor takes about one atomic a nanosecond, so a trip of fewer than
-// kSpFlush rows is staged in shared memory until that many are there: 15M
+// sp_flush rows is staged in shared memory until that many are there: 15M
 // rows with 9% matching, 12 rows a trip, were bound by the cursor (118 us).
-// Output order is arbitrary across warps.
-constexpr int kSpFlush = 64;
-constexpr int kSpStage = 2 * kSpFlush;  // rows staged at most: kSpFlush - 1 and one trip's
+// Output order is arbitrary across warps.  Trips of several items flush more
+// rows: at 64, 50M rows with 25% matching, 64 a trip of two items, took 280 us
+// against 235 without stages.
+template <int U>
+constexpr int sp_flush() { return U == 1 ? 64 : 96; }
+template <int U>
+constexpr int sp_stage() { return 2 * sp_flush<U>(); }  // rows staged at most: sp_flush - 1 and one trip's
 // REGS: 64 for one item, where the next trip's first column is loaded ahead
 // (50M rows, 1% kept by one filter: 226 us without stages and load, 74 with),
-// and for blocks past 512 threads, which launch with no more.  Two items hold
-// their loads in flight in up to 128 instead: at 64, with the load ahead, the
-// join and projection of 50M rows, 72% kept, took 442 us against 367.
+// and for blocks past 512 threads, which launch with no more.  More items hold
+// their loads in flight in up to 128 instead: two at 64, with the load ahead,
+// took 442 us against 367 for the join and projection of 50M rows, 72% kept.
 template <class SH, bool PRED, bool CHUNK, int U, int REGS>
 __global__ void __maxnreg__(REGS) k_project_sp(const __grid_constant__ KParams kp, const __grid_constant__ ProjOut out) {
   extern __shared__ float4 spmem[];
-  char* st = reinterpret_cast<char*>(spmem) + (threadIdx.x >> 5) * out_stage_bytes<SH, kSpStage>();
+  char* st = reinterpret_cast<char*>(spmem) + (threadIdx.x >> 5) * out_stage_bytes<SH, sp_stage<U>()>();
   bool overflow = false;
   int staged = 0;  // warp-uniform
   auto write_items = [&](Item<SH> (&it)[U]) {
@@ -268,16 +272,16 @@ __global__ void __maxnreg__(REGS) k_project_sp(const __grid_constant__ KParams k
     const int incl = warp_incl_scan(cnt);
     const int total = __shfl_sync(0xffffffffu, incl, 31);
     if (total == 0) return;
-    if (total < kSpFlush) {
+    if (total < sp_flush<U>()) {
       int slot = staged + incl - cnt;
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-          if ((it[u].mask >> r) & 1u) stage_out_row<SH, kSpStage>(st, slot++, it[u], r);
+          if ((it[u].mask >> r) & 1u) stage_out_row<SH, sp_stage<U>()>(st, slot++, it[u], r);
       staged += total;
-      if (staged >= kSpFlush) {
-        flush_out_rows<SH, kSpStage>(st, staged, out, overflow);
+      if (staged >= sp_flush<U>()) {
+        flush_out_rows<SH, sp_stage<U>()>(st, staged, out, overflow);
         staged = 0;
       }
       return;
@@ -298,7 +302,7 @@ __global__ void __maxnreg__(REGS) k_project_sp(const __grid_constant__ KParams k
       }
     }
   };
-  if constexpr (!PRED && !CHUNK && U != 2 && first_slot<SH>() >= 0) {
+  if constexpr (!PRED && !CHUNK && U == 1 && first_slot<SH>() >= 0) {
     for_items_ahead<SH, U>(kp, [&](Item<SH> (&it)[U], const int64_t (&idx)[U]) {
       eval_items<SH, false, U, true>(it, kp, idx);
       write_items(it);
@@ -310,7 +314,7 @@ __global__ void __maxnreg__(REGS) k_project_sp(const __grid_constant__ KParams k
       write_items(it);
     });
   }
-  if (staged > 0) flush_out_rows<SH, kSpStage>(st, staged, out, overflow);
+  if (staged > 0) flush_out_rows<SH, sp_stage<U>()>(st, staged, out, overflow);
   if (overflow) set_error(kp.err, PV_ERR_OUTPUT_OVERFLOW);
   __shared__ bool last;
   __syncthreads();
@@ -802,7 +806,7 @@ static pv_status launch_proj_sp(const LaunchCfg& c, const KParams& kp, const Pro
   auto k = k_project_sp<SH, P, C, U, U == 1 ? 64 : 128>;
   if constexpr (U == 2)
     if (c.block > 512) k = k_project_sp<SH, P, C, U, 64>;
-  const size_t smem = static_cast<size_t>(c.block / 32) * out_stage_bytes<SH, kSpStage>();
+  const size_t smem = static_cast<size_t>(c.block / 32) * out_stage_bytes<SH, sp_stage<U>()>();
   // the kernel's static shared memory counts too: 48 KB of stages (12-byte rows, 1024 threads) need the attribute
   if (smem >= 40 * 1024 &&
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
