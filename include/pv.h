@@ -472,9 +472,9 @@ pv_status pv_mlp_adam(pv_ctx* ctx, float* params, const float* grad, float* m, f
  * out_capacity) and *out_status (device int32) = PV_OK, or
  * PV_ERR_OUTPUT_OVERFLOW when more rows matched than fit.
  *
- * It allocates nothing: its scratch (an error word, a ticket and one word per
- * tile, about 0.5 MB) is one statically sized array in device memory that
- * every GPU loading this library holds until the process exits.  The first
+ * It allocates nothing: its scratch (an error word and match counts, about
+ * 0.15 MB) is one statically sized array in device memory that every GPU
+ * loading this library holds until the process exits.  The first
  * call on a device, with that device current, looks up the array's device
  * address (cudaGetSymbolAddress) and caches it; make that first call before
  * any stream capture.  Every call shares the one array and each clears what

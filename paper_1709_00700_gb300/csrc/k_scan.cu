@@ -5,8 +5,8 @@
 //   PROJECT multi pass (Section 4.1 fine-grained strategy: matches are
 //     counted, a prefix sum yields unique write positions, the matches are
 //     written in table order): matches are marked as bits and counted, then
-//     written; the allocation-free entry point does it in one kernel with a
-//     chained prefix sum.
+//     written; the allocation-free entry point has no room for the bits and
+//     filters again to write.
 #include <algorithm>
 #include <mutex>
 
@@ -331,7 +331,7 @@ __global__ void __maxnreg__(REGS) k_project_sp(const __grid_constant__ KParams k
   }
 }
 
-// Tile of the one-kernel ordered projection: blockDim * U items; its item of
+// Tile of the ordered projection without bits: blockDim * U items; its item of
 // (thread t, unroll u) is u * blockDim + t.
 template <int U>
 __device__ __forceinline__ void tile_items(int64_t tile, int64_t (&idx)[U]) {
@@ -403,7 +403,7 @@ __global__ void __maxnreg__(64) k_project_mark(const __grid_constant__ KParams k
       w |= __shfl_xor_sync(0xffffffffu, w, 1);
       w |= __shfl_xor_sync(0xffffffffu, w, 2);
       w |= __shfl_xor_sync(0xffffffffu, w, 4);
-      if ((lane & 7) == 0) out.bits[(unit * U + u) * 4 + (lane >> 3)] = w;
+      if (out.bits != nullptr && (lane & 7) == 0) out.bits[(unit * U + u) * 4 + (lane >> 3)] = w;
     }
     count = __reduce_add_sync(0xffffffffu, count);
     if (lane == 0 && count != 0) {
@@ -483,91 +483,20 @@ __global__ void __launch_bounds__(kMarkTileRows / 32) k_project_emit(const __gri
   }
 }
 
-// ---------------------------------------------------------------------------
-// Ordered projection in one pass, for the allocation-free entry point, which
-// has room for a word per tile but not for a bit per row.  CTAs take tiles in
-// order from a ticket counter; a tile's matches are counted and listed in
-// shared memory, its first output position is the sum of the counts of all
-// tiles before it (chained prefix sum with look-back, Merrill and Garland,
-// 2016), and the listed rows are then read and written one per lane.  Bound by
-// the latency of the look-back over the tiles in flight: 239 us for 50M rows
-// with 2% matching, against 264 us for counting, scanning and filtering again.
-// ---------------------------------------------------------------------------
-// Word of a tile: 0 (not counted yet), its count, or the count of all tiles up
-// to and including it; flag and value in one 64-bit word, so that one relaxed
-// access reads or publishes both.
-constexpr uint64_t kTileCount = 1ull << 62, kTilePrefix = 2ull << 62, kTileValue = kTileCount - 1;
-
-__device__ __forceinline__ uint64_t tile_word(const int64_t* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void tile_publish(int64_t* p, uint64_t v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(static_cast<unsigned long long>(v)) : "memory");
-}
-
-// Output position of a tile's first match (all lanes of one warp; the tile's
-// own count is published first).  Every tile before this one was taken by a
-// running CTA that publishes its count without waiting, so the wait ends;
-// after about two seconds it gives up all the same (PV_ERR_TIMEOUT, a base
-// past every capacity).
-__device__ __forceinline__ int64_t tile_base(int64_t* words, int64_t tile, int64_t count, int32_t* err) {
-  const int lane = threadIdx.x & 31;
-  if (lane == 0) tile_publish(words + tile, (tile == 0 ? kTilePrefix : kTileCount) | static_cast<uint64_t>(count));
-  if (tile == 0) return 0;
-  int64_t sum = 0;
-  uint64_t t0 = 0;
-  uint32_t polls = 0;
-  for (int64_t last = tile - 1;;) {  // lane l looks at tile last - l
-    const int64_t at = last - lane;
-    const uint64_t w = at >= 0 ? tile_word(words + at) : kTilePrefix;
-    const uint32_t prefix = __ballot_sync(0xffffffffu, (w >> 62) == 2);
-    const uint32_t unknown = __ballot_sync(0xffffffffu, (w >> 62) == 0);
-    const int stop = prefix ? __ffs(prefix) - 1 : 32;  // nearest tile whose prefix is known
-    const uint32_t upto = stop >= 31 ? 0xffffffffu : (2u << stop) - 1u;
-    if ((unknown & upto) == 0) {
-      sum += static_cast<int64_t>(
-          warp_reduce<PV_SUM>((upto >> lane) & 1u ? w & kTileValue : 0ull));
-      if (prefix) break;
-      last -= 32;
-      continue;
-    }
-    if ((++polls & 255u) == 0) {
-      uint64_t t;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      if (t0 == 0) t0 = t;
-      if (__any_sync(0xffffffffu, t - t0 > 2000000000ull)) {
-        if (lane == 0) {
-          set_error(err, PV_ERR_TIMEOUT);
-          tile_publish(words + tile, kTilePrefix | (kTileValue >> 1));
-        }
-        return static_cast<int64_t>(kTileValue >> 1);
-      }
-    }
-  }
-  if (lane == 0) tile_publish(words + tile, kTilePrefix | static_cast<uint64_t>(sum + count));
-  return sum;
-}
-
-// Rows of a tile at most: entries of its match list (16-bit row numbers).
-template <int U>
-constexpr int64_t tile_rows(int block) { return 4ll * block * U; }
-
-// Ticket and tile words start at zero (the launcher clears them): word -1 of
-// tile_count is the ticket.
+// Ordered projection without bits, for the allocation-free entry point, whose
+// static scratch holds the counts only: the second kernel filters its tile again.
+// One CTA per tile; the tile's matches become a row list in shared memory, and
+// the listed rows are read and written one per lane.  (One kernel with a chained
+// prefix sum, which filters once, is bound by its look-back: 1M rows took 18 us
+// against 15 by counting, scanning and filtering again, 10M 43 against 40.)
 template <class SH, int U>
-__global__ void __maxnreg__(64) k_project_ordered(const __grid_constant__ KParams kp,
-                                                  const __grid_constant__ ProjOut out) {
+__global__ void __maxnreg__(64) k_project_refilter(const __grid_constant__ KParams kp,
+                                                   const __grid_constant__ ProjOut out) {
   static_assert(U <= 4, "16-bit scan fields hold at most 4 unroll slots");
-  extern __shared__ uint16_t list[];  // tile rows that match, in output order
-  __shared__ int64_t s_tile, s_base;
-  unsigned long long* ticket = reinterpret_cast<unsigned long long*>(out.tile_count - 1);
-  for (;;) {
-    if (threadIdx.x == 0) s_tile = static_cast<int64_t>(atomicAdd(ticket, 1ull));
-    __syncthreads();
-    const int64_t tile = s_tile;
-    if (tile >= out.n_tiles) break;
+  __shared__ uint16_t list[kMarkTileRows];  // rows of the tile that match, in output order
+  pdl_wait();  // launched early behind the mark kernel
+  const int64_t n_tiles = mark_tiles(kp.n_rows);
+  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     int64_t idx[U];
     tile_items<U>(tile, idx);
     uint32_t mask[U];
@@ -578,8 +507,13 @@ __global__ void __maxnreg__(64) k_project_ordered(const __grid_constant__ KParam
 #pragma unroll
       for (int u = 0; u < U; ++u) mask[u] = it[u].mask;
     }
+    uint64_t before = 0, base;  // matches of earlier tiles
+    const int64_t super = tile >> out.mark_shift;
+    for (int64_t i = threadIdx.x; i < super; i += blockDim.x) before += out.mark_super[i];
+    for (int64_t i = (super << out.mark_shift) + threadIdx.x; i < tile; i += blockDim.x) before += out.mark_count[i];
+    block_excl_scan(before, &base);
     int total, pos[U];  // tile matches; list position of each item's first match
-    {  // row order inside the tile: (u, thread, row); one scan of U packed 16-bit counters (at most 4 * 1024 each)
+    {  // row order inside the tile: (u, thread, row); one scan of U packed 16-bit counters (at most 4 * 512 each)
       uint64_t packed = 0, t;
 #pragma unroll
       for (int u = 0; u < U; ++u) packed |= static_cast<uint64_t>(__popc(mask[u])) << (16 * u);
@@ -591,28 +525,15 @@ __global__ void __maxnreg__(64) k_project_ordered(const __grid_constant__ KParam
         total += static_cast<int>((t >> (16 * u)) & 0xFFFF);
       }
     }
-    const int64_t first_row = tile * tile_rows<U>(blockDim.x);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       int p = pos[u];
-      const uint16_t r0 = static_cast<uint16_t>(idx[u] * 4 - first_row);
+      const uint16_t r0 = static_cast<uint16_t>(idx[u] * 4 - tile * kMarkTileRows);
 #pragma unroll
       for (int r = 0; r < 4; ++r)
         if ((mask[u] >> r) & 1u) list[p++] = static_cast<uint16_t>(r0 + r);
     }
-    if (threadIdx.x < 32) {
-      const int64_t base = tile_base(out.tile_count, tile, total, kp.err);
-      if (threadIdx.x == 0) {
-        s_base = base;
-        if (tile == out.n_tiles - 1) {
-          const int64_t n = base + total;
-          *out.count = n < out.capacity ? n : out.capacity;
-          if (n > out.capacity) set_error(kp.err, PV_ERR_OUTPUT_OVERFLOW);
-        }
-      }
-    }
     __syncthreads();
-    const int64_t base = s_base;
     constexpr int K = 2;  // rows of a lane read together
     for (int i = threadIdx.x; i < total; i += K * blockDim.x) {
       Item<SH> it[K];
@@ -622,16 +543,21 @@ __global__ void __maxnreg__(64) k_project_ordered(const __grid_constant__ KParam
       for (int k = 0; k < K; ++k) {
         const int j = i + k * blockDim.x;
         has[k] = j < total;
-        rows[k] = first_row + (has[k] ? list[j] : 0);
+        rows[k] = tile * kMarkTileRows + (has[k] ? list[j] : 0);
       }
       compact_load_rows<SH, K, 1>(it, ok, kp, rows, has);
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        const int64_t p = base + i + k * blockDim.x;
-        if (ok[k] && p < out.capacity) write_row<SH>(out, it[k], 0, p);
+        const int64_t at = static_cast<int64_t>(base) + i + k * blockDim.x;
+        if (ok[k] && at < out.capacity) write_row<SH>(out, it[k], 0, at);
       }
     }
-    __syncthreads();  // the list and the shared words are free again
+    if (tile == n_tiles - 1 && threadIdx.x == 0) {
+      const int64_t n = static_cast<int64_t>(base) + total;
+      *out.count = n < out.capacity ? n : out.capacity;
+      if (n > out.capacity) set_error(kp.err, PV_ERR_OUTPUT_OVERFLOW);
+    }
+    __syncthreads();  // the list is free again
   }
 }
 
@@ -826,9 +752,12 @@ static pv_status launch_proj_sp(const LaunchCfg& c, const KParams& kp, const Pro
 // 10% matching: 72 us with one item, 37 with four; 100K rows 6.9 / 8.2).  A
 // tile is split until an SM has three units, at most into 8 (100K rows, all
 // matching: 14 us by whole tiles, 8 by counting twice).
+static bool mark_wide(const LaunchCfg& c, const KParams& kp) {
+  return kp.n_items >= static_cast<int64_t>(512) * c.sm_count;
+}
 template <class SH, bool P>
 static pv_status launch_proj_ordered(const LaunchCfg& c, const KParams& kp, const ProjOut& out) {
-  const bool wide = kp.n_items >= static_cast<int64_t>(512) * c.sm_count;
+  const bool wide = mark_wide(c, kp);
   auto km = wide ? k_project_mark<SH, P, 4> : k_project_mark<SH, P, 1>;
   auto ke = k_project_emit<SH>;
   LaunchCfg ce = c;
@@ -946,22 +875,25 @@ void register_scan_shapes() {
 }
 
 // ---------------------------------------------------------------------------
-// Allocation-free multi-pass projection (k_project_ordered: 256 threads, 4
-// items per thread, branched).  Its scratch -- the error word, the ticket and the
-// tile words -- lives in one file-scope device array instead of memory from an
-// allocator.  Every GPU that loads this library
-// holds the array until the process exits.
+// Allocation-free multi-pass projection (k_project_mark and k_project_refilter,
+// branched).  Its scratch -- the error word and the match counts per tile and
+// per super -- lives in one file-scope device array instead of memory from an
+// allocator.  Every GPU that loads this library holds the array until the
+// process exits.
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int kNoAllocBlock = 256;
+constexpr int kNoAllocBlock = 512;
 constexpr int kNoAllocU = 4;
-constexpr int64_t kNoAllocTileRows = 4LL * kNoAllocBlock * kNoAllocU;
-constexpr int64_t kNoAllocMaxTiles = (PV_NOALLOC_MAX_ROWS + kNoAllocTileRows - 1) / kNoAllocTileRows;
-constexpr int64_t kNoAllocHeader = 32;  // words: [0] error word (int32), [31] the ticket, rest unused padding
+static_assert(kNoAllocBlock * kNoAllocU * 4 == kMarkTileRows, "a CTA filters one tile");
+constexpr int64_t kNoAllocMaxTiles = (PV_NOALLOC_MAX_ROWS + kMarkTileRows - 1) / kMarkTileRows;
+constexpr int64_t kNoAllocHeader = 32;  // words: [0] error word (int32), rest unused padding
 
-// Scratch of every call: header, then the tile words.
-__device__ __align__(256) int64_t g_noalloc_scratch[kNoAllocHeader + kNoAllocMaxTiles];
+// Scratch of every call: header, then the supers (one per 16 tiles), then the
+// tiles' 32-bit counts.
+__device__ __align__(256) int64_t g_noalloc_scratch[kNoAllocHeader + kNoAllocMaxTiles / 16 + 1 +
+                                                    (kNoAllocMaxTiles + 1) / 2];
+static_assert(kNoAllocMaxTiles >> 4 <= 2048, "supers of 16 tiles at every row count");
 
 constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mu;
@@ -1033,22 +965,25 @@ extern "C" pv_status pv_filter_project_noalloc(const int32_t* a, const int32_t* 
   out.col[1] = out_price;
   out.capacity = out_capacity;
   out.count = out_count;
-  out.n_tiles = (kp.n_items + kNoAllocBlock * kNoAllocU - 1) / (kNoAllocBlock * kNoAllocU);
-  if (out.n_tiles < 1) out.n_tiles = 1;
-  out.tile_count = scratch + kNoAllocHeader;
-  // the array keeps the previous call's contents: clear the error word
-  if (cudaMemsetAsync(scratch, 0, sizeof(int32_t), s) != cudaSuccess) return PV_ERR_CUDA;
+  out.mark_shift = mark_shift(n_rows);
+  out.mark_super = reinterpret_cast<unsigned long long*>(scratch + kNoAllocHeader);
+  out.mark_count = reinterpret_cast<unsigned int*>(scratch + kNoAllocHeader + mark_super_bytes(n_rows) / 8);
   LaunchCfg c{};
   c.stream = s;
   c.sm_count = sms;
-  c.block = kNoAllocBlock;
-  auto k = k_project_ordered<ShFilterProj, kNoAllocU>;
-  const size_t smem = static_cast<size_t>(tile_rows<kNoAllocU>(c.block)) * sizeof(uint16_t);
-  const int grid = grid_for(c, reinterpret_cast<const void*>(k), smem, out.n_tiles, 1);
-  if (grid <= 0) return PV_ERR_UNSUPPORTED;
-  if (cudaMemsetAsync(out.tile_count - 1, 0, static_cast<size_t>(out.n_tiles + 1) * 8, s) != cudaSuccess)
-    return PV_ERR_CUDA;
-  k<<<grid, c.block, smem, s>>>(kp, out);
+  c.block = 256;
+  const bool wide = mark_wide(c, kp);
+  auto km = wide ? k_project_mark<ShFilterProj, false, 4> : k_project_mark<ShFilterProj, false, 1>;
+  auto ke = k_project_refilter<ShFilterProj, kNoAllocU>;
+  const int gm = grid_for(c, reinterpret_cast<const void*>(km), 0, kp.n_items, int64_t(c.block) * (wide ? 4 : 1));
+  LaunchCfg ce = c;
+  ce.block = kNoAllocBlock;
+  const int ge = grid_for(ce, reinterpret_cast<const void*>(ke), 0, mark_tiles(n_rows), 1);
+  if (gm <= 0 || ge <= 0) return PV_ERR_UNSUPPORTED;
+  // the array keeps the previous call's contents: clear the error word and the counts
+  if (cudaMemsetAsync(scratch, 0, kNoAllocHeader * 8 + mark_count_bytes(n_rows), s) != cudaSuccess) return PV_ERR_CUDA;
+  km<<<gm, c.block, 0, s>>>(kp, out);
+  if (pdl_launch(ke, dim3(ge), dim3(kNoAllocBlock), 0, s, kp, out) != cudaSuccess) return PV_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return PV_ERR_CUDA;
   if (cudaMemcpyAsync(out_status, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return PV_ERR_CUDA;

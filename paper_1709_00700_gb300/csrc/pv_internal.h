@@ -83,8 +83,7 @@ struct ProjOut {
   unsigned long long* cursor;   // single pass: write cursor (zero between runs)
   int64_t* count;               // rows written (min(total, capacity))
   unsigned int* done;           // block ticket (zero between runs)
-  int64_t* tile_count;          // multi pass, generic kernels: matches per tile (allocation-free entry
-                                // point: tile words, the word before them is the ticket)
+  int64_t* tile_count;          // multi pass, generic kernels: matches per tile
   int64_t* tile_offset;         // multi pass, generic kernels: exclusive prefix of tile_count
   int64_t n_tiles;
   // multi pass, compiled shapes: matches per 2^mark_shift tiles (the counts of the tiles follow), one bit
