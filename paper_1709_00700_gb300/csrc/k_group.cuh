@@ -978,6 +978,7 @@ static pv_status launch_k(const LaunchCfg& c, K k, const KParams& kp, const Grou
   }
   const int grid = grid_for(c, reinterpret_cast<const void*>(k), smem, kp.n_items, static_cast<int64_t>(c.block) * U);
   if (grid <= 0) return PV_ERR_UNSUPPORTED;
+  if (c.check) return PV_OK;
   // rows one thread visits, at most: its items (grid-stride, chunked or staged) of 4 rows, or for
   // compacted execution as many queued rows, plus one partial drain
   const int64_t T = static_cast<int64_t>(grid) * c.block;
@@ -1138,16 +1139,20 @@ template <class SH, int UMASK>
 static pv_status launch_group(const LaunchCfg& c, const KParams& kp, const GroupDesc& gd, const GroupOut& g0,
                               const PartOut& po, const pv_variant& v) {
   GroupOut g = g0;
-  if (po.key != nullptr) {
-    if constexpr (part_hash_ok<SH>()) {
-      if (g.ht == PV_HT_LINEAR) {
-        const pv_status s = run_part<SH, true>(c, kp, gd, g, po);
+  if constexpr (part_perfect_ok<SH>()) {
+    if (po.key != nullptr) {
+      // A variant that the general kernels refuse is refused here, with nothing enqueued.
+      LaunchCfg check = c;
+      check.check = true;
+      pv_status s = g.ht == PV_HT_LINEAR ? run_group<SH, UMASK, SinkGInsert>(check, kp, gd, g, 0)
+                                         : run_group<SH, UMASK, SinkGlobalPerfect>(check, kp, gd, g, 0);
+      if (s != PV_OK) return s;
+      if (g.ht == PV_HT_PERFECT) return run_part<SH, false>(c, kp, gd, g, po);
+      if constexpr (part_hash_ok<SH>()) {
+        s = run_part<SH, true>(c, kp, gd, g, po);
         if (s != PV_OK) return s;
         g.guard = po.ctl + kPartCtlFull;  // the general kernels below run when a range was full
       }
-    }
-    if constexpr (part_perfect_ok<SH>()) {
-      if (g.ht == PV_HT_PERFECT) return run_part<SH, false>(c, kp, gd, g, po);
     }
   }
   const bool multi = v.exec == PV_EXEC_MULTI_PASS;

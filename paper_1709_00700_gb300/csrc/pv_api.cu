@@ -1098,6 +1098,7 @@ pv_status pv_run_pipeline(pv_ctx* c, const pv_pipeline_spec* spec, const pv_vari
   s = alloc_result(c, *r);
   if (s == PV_OK) s = launch_result(c, *r);
   if (s != PV_OK) {
+    cudaStreamSynchronize(c->stream);  // what was enqueued so far (the tables' clears) writes the memory
     for (void* p : r->mem) dfree(c, p);
     return s;
   }

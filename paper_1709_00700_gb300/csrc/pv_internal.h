@@ -33,6 +33,7 @@ struct LaunchCfg {
   bool staged;    // TMA-staged access (grouped predicated pipelines)
   int compact_probes;  // compacted: probes of the first stage (1 or 2)
   int first_items;     // compacted: items a lane takes through the first stage per trip (1 or 2)
+  bool check;     // grouped: only tell whether the variant's kernels can be launched
   int* launches;  // incremented per kernel launch
   // optional per-kernel timing: called right before and right after a launch
   void (*mark)(void* timer, cudaStream_t s);
