@@ -78,6 +78,7 @@ struct Column {
   int64_t n_rows;                          // rows; for a result column its capacity
   bool has_stats = false;
   int64_t vmin = 0, vmax = 0;
+  int32_t top = 0;                         // of kSampleRows sampled rows, those of the commonest value (0: unknown)
   const unsigned long long* n_dyn = nullptr;  // result column: row count on the device
   int32_t src_res = 0;                     // result column: the result it belongs to
 };
@@ -498,6 +499,34 @@ __global__ void k_minmax(const T* p, int64_t n, const unsigned long long* n_dyn,
   }
 }
 
+// Skew of a key column: of kSampleRows rows at hashed positions (evenly spaced ones could meet a period of the
+// data), how many hold the commonest value.  One CTA counts them in shared memory.
+constexpr int kSampleRows = 1024;
+template <class T>
+__global__ void __launch_bounds__(kSampleRows) k_sample_top(const T* p, int64_t n, unsigned long long* out) {
+  constexpr uint32_t S = 2 * kSampleRows;  // slots
+  __shared__ unsigned long long key[S];
+  __shared__ unsigned int count[S];
+  __shared__ unsigned int top;
+  for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) {
+    key[i] = kEmpty64;
+    count[i] = 0;
+  }
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  const int64_t row = static_cast<int64_t>(__umul64hi(fmix64(threadIdx.x + 1), static_cast<uint64_t>(n)));
+  const unsigned long long v = static_cast<uint32_t>(p[row]);
+  uint32_t s = static_cast<uint32_t>(fmix64(v)) & (S - 1);
+  for (uint32_t step = 0; step < S; ++step) {
+    const unsigned long long cur = atomicCAS(key + s, kEmpty64, v);
+    if (cur == kEmpty64 || cur == v) break;
+    s = (s + 1) & (S - 1);
+  }
+  atomicMax(&top, atomicAdd(count + s, 1u) + 1u);
+  __syncthreads();
+  if (threadIdx.x == 0) *out = top;
+}
+
 __global__ void k_flush(uint4* p, int64_t n, uint32_t salt) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     p[i] = make_uint4(salt, (uint32_t)i, salt ^ 0x9e3779b9u, (uint32_t)(i >> 32));
@@ -588,17 +617,19 @@ static pv_status column_stats(pv_ctx* c, pv_col h, int64_t* mn, int64_t* mx) {
   if (!col.has_stats) {
     if (c->capturing) return fail(c, PV_ERR_INVALID_ARG, "column statistics needed while capturing");
     unsigned long long* d = reinterpret_cast<unsigned long long*>(c->d_stats);
-    PV_CUDA(c, cudaMemsetAsync(d, 0, 16, c->stream));
+    PV_CUDA(c, cudaMemsetAsync(d, 0, 24, c->stream));
     const int grid = std::max(1, std::min<int>(c->sm_count * 4, static_cast<int>((col.n_rows + 255) / 256)));
     if (col.n_rows > 0) {
       const unsigned long long* nd = col.n_dyn;
       if (col.type == PV_I32) k_minmax<<<grid, 256, 0, c->stream>>>(static_cast<const int32_t*>(col.ptr), col.n_rows, nd, d);
       else if (col.type == PV_I64) k_minmax<<<grid, 256, 0, c->stream>>>(static_cast<const int64_t*>(col.ptr), col.n_rows, nd, d);
       else k_minmax<<<grid, 256, 0, c->stream>>>(static_cast<const uint8_t*>(col.ptr), col.n_rows, nd, d);
+      if (col.type == PV_I32 && nd == nullptr && col.n_rows >= kPartMinRows)
+        k_sample_top<<<1, kSampleRows, 0, c->stream>>>(static_cast<const int32_t*>(col.ptr), col.n_rows, d + 2);
       PV_CUDA(c, cudaGetLastError());
     }
-    unsigned long long hbuf[2] = {0, 0};
-    PV_CUDA(c, cudaMemcpyAsync(hbuf, d, 16, cudaMemcpyDeviceToHost, c->stream));
+    unsigned long long hbuf[3] = {0, 0, 0};
+    PV_CUDA(c, cudaMemcpyAsync(hbuf, d, 24, cudaMemcpyDeviceToHost, c->stream));
     PV_CUDA(c, cudaStreamSynchronize(c->stream));
     // some row was present: a row's max code and min code are not both 0 (that would need the
     // value to be INT64_MIN and INT64_MAX at once)
@@ -609,6 +640,7 @@ static pv_status column_stats(pv_ctx* c, pv_col h, int64_t* mn, int64_t* mx) {
       col.vmin = 0;
       col.vmax = -1;
     }
+    col.top = static_cast<int32_t>(hbuf[2]);
     col.has_stats = true;
   }
   *mn = col.vmin;
@@ -617,9 +649,54 @@ static pv_status column_stats(pv_ctx* c, pv_col h, int64_t* mn, int64_t* mx) {
 }
 
 
-// Scratch for the partitioned aggregation (k_part.cuh) of a result whose table
-// is global and too large to be updated in place cheaply; without it (not the
-// variant, too few rows, no memory) the general kernels run.
+// Whether the partitioned kernels (k_part.cuh) are the faster ones for a result with a global table, and never
+// much the slower: they read the key twice and write and read a record for every row that passes, whatever the
+// table; the general kernels pay for each such row by where the table is and how its rows collide.  Measured as
+// general / partitioned in us, SUM and COUNT by an int32 key.  `keep` is the share of rows that pass the filters,
+// by their ranges and the columns' minima and maxima; `hot` whether one key holds a 64th of the rows or more.
+static bool part_pays(pv_ctx* c, const Result& r) {
+  const Canon& k = r.canon;
+  const GroupOut& g = r.grp;
+  const int64_t n = k.n_rows;
+  const bool hash = g.ht == PV_HT_LINEAR, filtered = k.gs.n_preds > 0;
+  if (n < kPartMinRows || n > (int64_t(1) << 31) || (!hash && g.cap < kPartMinSlots)) return false;
+  double keep = 1.0, hot_share = 1.0;
+  for (int i = 0; i < k.gs.n_preds; ++i) {
+    int64_t mn, mx;
+    if (column_stats(c, k.slot_col[k.gs.pred_slot[i]], &mn, &mx) != PV_OK) return false;
+    const double lo = static_cast<double>(std::max(k.kp.lo[i], mn)), hi = static_cast<double>(std::min(k.kp.hi[i], mx));
+    keep *= hi < lo ? 0.0 : (hi - lo + 1) / (static_cast<double>(mx) - static_cast<double>(mn) + 1);
+  }
+  for (int i = 0; i < k.n_keys; ++i) hot_share *= static_cast<double>(c->cols[k.key_src[i][0]].top) / kSampleRows;
+  const bool hot = hot_share >= 1.0 / 64;
+  const int64_t bytes = g.cap * (g.stride + (hash ? 1 : 0)) * 8;
+  const bool large = bytes >= (int64_t(16) << 20), far = bytes > c->l2_bytes;
+  const int64_t M = int64_t(1) << 20;
+  if (hash) {
+    // 300K and 1M groups: all of 1.1M uniform rows 62 / 56, 102 / 62, 30% 59 / 59, 81 / 62, 10% 44 / 57, 59 / 60
+    if (n < 4 * M) return large && keep >= 0.3;
+    if (hot) return keep >= (n < 16 * M ? 0.3 : 0.01);  // 4.3M rows, 30K groups: 30% 174 / 101, 10% 85 / 94
+    // 4.3M uniform rows, 300K groups: 30% 127 / 97, 90% 128 / 133, all 119 / 131; 1M groups all 215 / 147
+    if (n < 16 * M) return large && keep >= 0.3 && (filtered || bytes >= (int64_t(48) << 20));
+    // 60M uniform rows: 300K groups 1% 1000 / 432, 30% 1382 / 835, 90% 1445 / 1323, all 1092 / 1113; all of 1000
+    // groups 2125 / 1580
+    return filtered ? keep >= 0.01 : far || g.cap <= (int64_t(1) << 12);
+  }
+  // 60M rows, 1e7 groups, far: all 2342 / 650, 30% 967 / 743, 10% 547 / 641; three key parts, 9.3M slots 2407 / 1091
+  if (far && keep >= 0.2) return true;
+  // skewed keys: all of 1.1M rows, 4200 groups 164 / 34; 30% of 1.1M rows, 1e5 groups 74 / 40, 10% 31 / 38; 10% of
+  // 4.3M rows 96 / 63; 1% of 60M rows 253 / 415
+  if (hot && keep >= (n < 4 * M ? 0.3 : 0.1)) return true;
+  // few slots and many rows, which collide: 17M rows, 4200 groups 394 / 178, 90% 359 / 263, 30% 137 / 194; 1e4
+  // groups 242 / 178, 90% 220 / 263; three key parts, 4913 slots 348 / 282, 216K slots 207 / 317
+  if (n >= 16 * M && g.cap <= (filtered ? int64_t(1) << 13 : int64_t(1) << 14) && keep >= 0.8) return true;
+  // a large table in L2: 1e6 groups, all of 1.1M rows 42 / 34, of 60M 672 / 641, 90% of 60M 620 / 956; three key
+  // parts, 60M rows, 2.2M slots 772 / 1111
+  return large && !filtered && k.n_keys == 1;
+}
+
+// Scratch for the partitioned aggregation of a result; without it (not the variant, not the faster way, no memory)
+// the general kernels run.
 static void alloc_part(pv_ctx* c, Result& r) {
   const Canon& k = r.canon;
   const GroupOut& g = r.grp;
@@ -630,16 +707,7 @@ static void alloc_part(pv_ctx* c, Result& r) {
   const bool hash = g.ht == PV_HT_LINEAR;
   if (hash ? !r.entry->part_hash : g.ht != PV_HT_PERFECT) return;
   const int words = r.entry->part_words;
-  // Where the partitioned kernels are the faster ones (us, general kernels against partitioned): atomics on
-  // tables past 16 MB (1.1M rows, 1e6 groups 43 / 34; 4M rows, 1e7 groups 395 / 112); many rows (20M rows, 1e4
-  // groups 284 / 205; hash table of 3e4 groups 568 / 397); skew, which a perfect array's variant states with
-  // warp_agg (1.1M rows, 1e5 groups 140 / 33).  A small table with fewer rows stays with the general
-  // kernels (4M rows, 1e5 groups 49 / 76).
-  const bool big = g.cap * (g.stride + (hash ? 1 : 0)) * 8 >= (int64_t(16) << 20);
-  const bool many = k.n_rows >= (hash ? int64_t(4) << 20 : int64_t(16) << 20);
-  if (k.n_rows < kPartMinRows || k.n_rows > (int64_t(1) << 31) || (!hash && g.cap < kPartMinSlots) ||
-      !(big || many || (!hash && v.warp_agg)))
-    return;
+  if (!part_pays(c, r)) return;
   // about 600 ranges of a perfect array (fewer leave SMs idle, more shorten the runs the scatter writes: 60M
   // rows in 391 ranges 334 us, in 1221 498 us), about 1024 of a hash table (smaller ranges spread hot keys),
   // of at least 256 slots, at most what an SM's shared memory holds
