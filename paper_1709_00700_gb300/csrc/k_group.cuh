@@ -1241,7 +1241,7 @@ static void reg_grouped() {
   e.sig = SH::signature();
   e.mode = MODE_GROUPED;
   e.grouped = launch_group<SH, UMASK>;
-  e.part_words = part_perfect_ok<SH>() ? part_words<typename SH::Aggs>() : -1;
+  e.part_perfect = part_perfect_ok<SH>();
   e.part_hash = part_hash_ok<SH>();
   register_shape(e);
 }

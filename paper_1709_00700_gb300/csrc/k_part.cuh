@@ -7,13 +7,14 @@
 //                   counts into row offsets and into units of at most
 //                   unit_rows rows, so that a hot range is shared by CTAs;
 //   k_part_scatter  sorts tiles of rows by range in shared memory and appends
-//                   each range's run to the range (key, aggregate codes);
+//                   each range's run to the range (group and value);
 //   k_part_agg      takes a unit at a time into a shared-memory table and
 //                   writes its groups straight to the result columns.  The
 //                   units of a shared range add into the range's slots of the
 //                   global table, which the last one extracts and empties.
-// The bytes: the key twice and the values once from the table, one write and
-// one read of (4 + 8 * values) bytes a row, each group once.  60M rows of an
+// A record is the row's group (key or slot) and the value of its SUM: 12 bytes.
+// The bytes: the key twice and the value once from the table, one write and one
+// read of a record a row, each group once.  60M rows of an
 // int32 key with 1e7 groups and an int64 value took 2041 us of atomics and
 // 312 us of extraction; they take 57 + 373 + 233 us.  The count reads at 0.6 of
 // the copy rate; the scatter is bound by the latency of its phases (a tile of
@@ -31,34 +32,25 @@ constexpr int kPartBlock = 512;
 constexpr int kPartMax = kPartMaxRanges;  // two words each in the scatter's shared memory
 constexpr uint32_t kPartNone = 0xFFFFFFFFu;
 
-// Value words of a record: one per aggregate that is not COUNT.
+// The aggregate of a record's value: the one SUM of a shape whose other
+// aggregates are COUNTs (-1: another shape).
 template <class A>
-constexpr int part_words() {
-  int n = 0;
-  for (int i = 0; i < A::N; ++i) n += A::func_of[i] != PV_COUNT;
-  return n;
-}
-// Value word of aggregate i (-1: COUNT).
-template <class A>
-constexpr int part_word(int i) {
-  int n = 0;
-  for (int j = 0; j < i; ++j) n += A::func_of[j] != PV_COUNT;
-  return A::func_of[i] == PV_COUNT ? -1 : n;
-}
-// Aggregate of value word w.
-template <class A>
-constexpr int part_agg(int w) {
-  for (int i = 0; i < A::N; ++i)
-    if (part_word<A>(i) == w) return i;
-  return 0;
+constexpr int part_sum() {
+  int at = -1;
+  for (int i = 0; i < A::N; ++i) {
+    if (A::func_of[i] == PV_COUNT) continue;
+    if (A::func_of[i] != PV_SUM || at >= 0) return -1;
+    at = i;
+  }
+  return at;
 }
 
-// Shapes with partitioned kernels: no probes (they would run twice), at most two
-// value words a record, keys of 32-bit parts (a perfect array's slot number is
-// the record's key; a hash table's key must itself be 32 bits).
+// Shapes with partitioned kernels: one SUM, no probes (they would run twice),
+// keys of 32-bit parts (a perfect array's slot number is the record's group; a
+// hash table's key must itself be 32 bits).
 template <class SH>
 constexpr bool part_perfect_ok() {
-  return SH::Probes::N == 0 && part_words<typename SH::Aggs>() <= kPartWords && key_narrow<SH>();
+  return SH::Probes::N == 0 && part_sum<typename SH::Aggs>() >= 0 && key_narrow<SH>();
 }
 template <class SH>
 constexpr bool part_hash_ok() { return part_perfect_ok<SH>() && SH::Key::N == 1; }
@@ -196,14 +188,11 @@ __global__ void __launch_bounds__(kPartBlock) k_part_hist(const __grid_constant_
   pdl_launch_dependents();
 }
 
-// Tile of the scatter: 8192 rows (4096 with two value words): runs of several
-// rows per range even at 2048 ranges, two CTAs per SM.
-template <class SH>
-constexpr int part_items() { return part_words<typename SH::Aggs>() <= 1 ? 4 : 2; }
-template <class SH>
-constexpr size_t part_scatter_smem(int n_parts) {
-  return static_cast<size_t>(kPartBlock) * 4 * part_items<SH>() * (8 * part_words<typename SH::Aggs>() + 4) +
-         2 * sizeof(uint32_t) * n_parts;
+// Tile of the scatter: 8192 rows, so that runs have several rows per range even
+// at 2048 ranges, and two CTAs fit an SM.
+constexpr int kPartItems = 4;  // per thread
+inline size_t part_scatter_smem(int n_parts) {
+  return static_cast<size_t>(kPartBlock) * 4 * kPartItems * 12 + 2 * sizeof(uint32_t) * n_parts;
 }
 
 template <class SH, bool HASH>
@@ -214,12 +203,12 @@ __global__ void __launch_bounds__(kPartBlock, 2) k_part_scatter(const __grid_con
   using KS = PartKeyShape<SH>;
   using VS = PartValShape<SH>;
   using A = typename SH::Aggs;
-  constexpr int U = part_items<SH>();
-  constexpr int NV = part_words<A>();
+  using Sum = typename At<part_sum<A>(), typename A::L>::type;
+  constexpr int U = kPartItems;
   constexpr int TR = kPartBlock * 4 * U;
   extern __shared__ unsigned long long smem[];
-  unsigned long long* sval = smem;                                // [NV][TR]
-  uint32_t* skey = reinterpret_cast<uint32_t*>(smem + NV * TR);   // [TR]
+  unsigned long long* sval = smem;                           // [TR]
+  uint32_t* skey = reinterpret_cast<uint32_t*>(smem + TR);   // [TR]
   uint32_t* start = skey + TR;                                    // rows of a range, then its first row in the tile
   uint32_t* delta = start + po.n_parts;                           // range's next output row - first row in the tile
   pdl_wait();
@@ -335,11 +324,7 @@ __global__ void __launch_bounds__(kPartBlock, 2) k_part_scatter(const __grid_con
           const uint32_t pos =
               start[part_of(key[h + u][r])] + ((rank[h + u][r >> 1] >> (16 * (r & 1))) & 0xFFFFu);
           skey[pos] = key[h + u][r];
-          static_for<NV>([&](auto w) {
-            constexpr int W = decltype(w)::value;
-            using AG = typename At<part_agg<A>(W), typename A::L>::type;
-            sval[W * TR + pos] = acc_code<AG::func>(agg_value<AG>(vals[u], kp, r));
-          });
+          sval[pos] = static_cast<unsigned long long>(agg_value<Sum>(vals[u], kp, r));
         }
     }
 #pragma unroll
@@ -355,8 +340,7 @@ __global__ void __launch_bounds__(kPartBlock, 2) k_part_scatter(const __grid_con
       const uint32_t k = skey[i];
       const uint32_t to_row = delta[part_of(k)] + i;
       po.key[to_row] = k;
-#pragma unroll
-      for (int w = 0; w < NV; ++w) po.val[w][to_row] = sval[w * TR + i];
+      po.val[to_row] = sval[i];
     }
     __syncthreads();
   }
@@ -364,27 +348,21 @@ __global__ void __launch_bounds__(kPartBlock, 2) k_part_scatter(const __grid_con
 }
 
 // Shared memory of k_part_agg: per slot (and one side slot for the hash key
-// equal to the empty marker) the value words, the row count, the hash key.
-inline size_t part_agg_smem(int words, bool hash, int shift) {
+// equal to the empty marker) the sum, the row count, the hash key.
+inline size_t part_agg_smem(bool hash, int shift) {
   const size_t s = (size_t{1} << shift) + 2;
-  return s * (8 * words + 4 + (hash ? 4 : 0));
+  return s * (8 + 4 + (hash ? 4 : 0));
 }
 
 // Result row of slot `key` of a perfect array, or of hash key `key`.
 template <class SH, bool HASH>
 __device__ __forceinline__ void part_write_group(const GroupDesc& gd, const GroupOut& g, int64_t pos, uint32_t key,
-                                                 const unsigned long long (&v)[part_words<typename SH::Aggs>() + 1],
-                                                 uint64_t count) {
+                                                 unsigned long long sum, uint64_t count) {
   using A = typename SH::Aggs;
   write_keys(gd, g, pos, !HASH, key);
   static_for<A::N>([&](auto a) {
     constexpr int I = decltype(a)::value;
-    constexpr int W = part_word<A>(I);
-    constexpr int F = A::func_of[I];
-    int64_t x;
-    if constexpr (W < 0) x = static_cast<int64_t>(count);
-    else x = decode_agg(F, v[W < 0 ? 0 : W]);
-    g.out[(SH::Key::N + I) * g.out_cap + pos] = x;
+    g.out[(SH::Key::N + I) * g.out_cap + pos] = static_cast<int64_t>(I == part_sum<A>() ? sum : count);
   });
 }
 
@@ -393,20 +371,19 @@ __global__ void __launch_bounds__(1024) k_part_agg(const __grid_constant__ KPara
                                                             const __grid_constant__ GroupDesc gd,
                                                             const __grid_constant__ GroupOut g,
                                                             const __grid_constant__ PartOut po) {
-  using A = typename SH::Aggs;
-  constexpr int NV = part_words<A>();
+  constexpr int kSum = part_sum<typename SH::Aggs>();  // the sum's word of a global slot
   extern __shared__ unsigned long long smem[];
   const uint32_t S = 1u << po.shift;
   const uint32_t SS = S + 2;  // slot S: the side slot
-  unsigned long long* sval = smem;                                // [NV][SS]
-  uint32_t* scnt = reinterpret_cast<uint32_t*>(smem + NV * SS);   // [SS]
-  uint32_t* skey = scnt + SS;                                     // [SS], hash only
+  unsigned long long* sval = smem;                           // [SS]
+  uint32_t* scnt = reinterpret_cast<uint32_t*>(smem + SS);   // [SS]
+  uint32_t* skey = scnt + SS;                                // [SS], hash only
   __shared__ uint32_t s_unit, s_part, s_last;
   __shared__ unsigned long long s_base;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t warps = blockDim.x >> 5;
   // One row (or a warp's rows of one key) into the table.
-  auto add = [&](uint32_t k, const unsigned long long (&v)[NV + 1], uint32_t count) {
+  auto add = [&](uint32_t k, unsigned long long v, uint32_t count) {
     uint32_t s = k & (S - 1);
     if constexpr (HASH) {
       if (k == kPartNone) {
@@ -427,21 +404,12 @@ __global__ void __launch_bounds__(1024) k_part_agg(const __grid_constant__ KPara
       }
     }
     atomicAdd(scnt + s, count);
-    static_for<NV>([&](auto w) {
-      constexpr int W = decltype(w)::value;
-      constexpr int F = A::func_of[part_agg<A>(W)];
-      unsigned long long* p = sval + W * SS + s;
-      if constexpr (F == PV_SUM) {
-        shared_add64(p, v[W]);
-      } else if (*reinterpret_cast<volatile unsigned long long*>(p) < v[W]) {
-        atomicMax(p, v[W]);
-      }
-    });
+    shared_add64(sval + s, v);
   };
   pdl_wait();
   for (;;) {
     if (threadIdx.x == 0) s_unit = atomicAdd(po.ctl + kPartCtlUnit, 1u);
-    for (uint32_t i = threadIdx.x; i < NV * SS; i += blockDim.x) sval[i] = 0;
+    for (uint32_t i = threadIdx.x; i < SS; i += blockDim.x) sval[i] = 0;
     for (uint32_t i = threadIdx.x; i < SS; i += blockDim.x) {
       scnt[i] = 0;
       if constexpr (HASH) skey[i] = kPartNone;
@@ -465,19 +433,17 @@ __global__ void __launch_bounds__(1024) k_part_agg(const __grid_constant__ KPara
         if (f < r1) {
           const uint32_t n = min(r1 - f, b == r0 ? ahead : trip);
           part_prefetch(po.key, f, n);
-#pragma unroll
-          for (int w = 0; w < NV; ++w) part_prefetch(po.val[w], f, n);
+          part_prefetch(po.val, f, n);
         }
       }
       uint32_t k[K];
-      unsigned long long v[K][NV + 1];
+      unsigned long long v[K];
 #pragma unroll
       for (int j = 0; j < K; ++j) {
         const uint32_t r = b + lane + j * blockDim.x;
         const bool in = r < r1;
         k[j] = in ? __ldcs(po.key + r) : 0u;
-#pragma unroll
-        for (int w = 0; w < NV; ++w) v[j][w] = in ? __ldcs(po.val[w] + r) : 0ull;
+        v[j] = in ? __ldcs(po.val + r) : 0ull;
       }
 #pragma unroll
       for (int j = 0; j < K; ++j) {
@@ -491,11 +457,7 @@ __global__ void __launch_bounds__(1024) k_part_agg(const __grid_constant__ KPara
             const uint32_t same = __ballot_sync(0xffffffffu, mine && k[j] == hk);
             if (__popc(same) < 8) continue;
             const bool peer = mine && k[j] == hk;
-            unsigned long long s[NV + 1];
-            static_for<NV>([&](auto w) {
-              constexpr int W = decltype(w)::value;
-              s[W] = warp_reduce<A::func_of[part_agg<A>(W)]>(peer ? v[j][W] : 0ull);
-            });
+            const unsigned long long s = warp_reduce<PV_SUM>(peer ? v[j] : 0ull);
             if (lane == 0) add(hk, s, __popc(same));
             mine = mine && !peer;
           }
@@ -531,12 +493,7 @@ __global__ void __launch_bounds__(1024) k_part_agg(const __grid_constant__ KPara
         }
         unsigned long long* dst = g.vals + slot * g.stride;
         atomicAdd(dst + gd.count_word, static_cast<unsigned long long>(count));
-        static_for<NV>([&](auto w) {
-          constexpr int W = decltype(w)::value;
-          constexpr int I = part_agg<A>(W);
-          const unsigned long long x = sval[W * SS + i];
-          if (x) acc_atomic<A::func_of[I]>(dst + I, x);
-        });
+        if (sval[i]) atomicAdd(dst + kSum, sval[i]);
       }
       __threadfence();
       __syncthreads();
@@ -570,26 +527,22 @@ __global__ void __launch_bounds__(1024) k_part_agg(const __grid_constant__ KPara
         const int64_t at = pos + __popc(ball & ((1u << lane) - 1u));
         pos += __popc(ball);
         if (occ) {
-          unsigned long long v[NV + 1];
+          unsigned long long sum;
           uint64_t count;
           uint32_t key = static_cast<uint32_t>(slot0) + i;
           if (units == 1) {
             count = scnt[i];
-#pragma unroll
-            for (int w = 0; w < NV; ++w) v[w] = sval[w * SS + i];
+            sum = sval[i];
             if constexpr (HASH) key = i == S ? kPartNone : skey[i];
           } else {
             unsigned long long* src = g.vals + (slot0 + i) * g.stride;
             count = __ldcg(src + gd.count_word);
-            static_for<NV>([&](auto w) {
-              constexpr int W = decltype(w)::value;
-              v[W] = __ldcg(src + part_agg<A>(W));
-            });
+            sum = __ldcg(src + kSum);
             if constexpr (HASH) key = static_cast<uint32_t>(__ldcg(g.keys + slot0 + i));
             for (int a = 0; a <= gd.n_aggs; ++a) src[a] = 0;
             if constexpr (HASH) g.keys[slot0 + i] = kEmpty64;
           }
-          if (at < g.out_cap) part_write_group<SH, HASH>(gd, g, at, key, v, count);
+          if (at < g.out_cap) part_write_group<SH, HASH>(gd, g, at, key, sum, count);
         }
       }
     }
@@ -607,14 +560,13 @@ static pv_status run_part(const LaunchCfg& c, const KParams& kp, const GroupDesc
   auto kh = k_part_hist<SH, HASH>;
   auto ks = k_part_scatter<SH, HASH>;
   auto ka = k_part_agg<SH, HASH>;
-  const size_t ssmem = part_scatter_smem<SH>(po.n_parts);
-  const size_t asmem = part_agg_smem(part_words<typename SH::Aggs>(), HASH, po.shift);
+  const size_t ssmem = part_scatter_smem(po.n_parts);
+  const size_t asmem = part_agg_smem(HASH, po.shift);
   if (cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(ssmem)) != cudaSuccess ||
       cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(asmem)) != cudaSuccess)
     return PV_ERR_CUDA;
-  constexpr int U = part_items<SH>();
   const int gh = grid_for(cp, reinterpret_cast<const void*>(kh), 0, kp.n_items, kPartBlock * 4);
-  const int gs = grid_for(cp, reinterpret_cast<const void*>(ks), ssmem, kp.n_items, kPartBlock * U);
+  const int gs = grid_for(cp, reinterpret_cast<const void*>(ks), ssmem, kp.n_items, kPartBlock * kPartItems);
   LaunchCfg ca = cp;
   ca.block = asmem > (size_t{110} << 10) ? 1024 : kPartBlock;  // a table that leaves room for one CTA on an SM
   const int ga = grid_for(ca, reinterpret_cast<const void*>(ka), asmem, kp.n_rows / po.unit_rows + po.n_parts, 1);

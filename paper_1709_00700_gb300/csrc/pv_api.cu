@@ -701,17 +701,16 @@ static void alloc_part(pv_ctx* c, Result& r) {
   const Canon& k = r.canon;
   const GroupOut& g = r.grp;
   const pv_variant& v = r.var;
-  if (r.generic || !r.entry || r.entry->part_words < 0 || v.agg != PV_AGG_GLOBAL || v.exec != PV_EXEC_SINGLE_PASS ||
+  if (r.generic || !r.entry || !r.entry->part_perfect || v.agg != PV_AGG_GLOBAL || v.exec != PV_EXEC_SINGLE_PASS ||
       v.threads_per_table == 1 || v.pred == PV_COMPACTED || v.access == PV_STAGED)
     return;
   const bool hash = g.ht == PV_HT_LINEAR;
   if (hash ? !r.entry->part_hash : g.ht != PV_HT_PERFECT) return;
-  const int words = r.entry->part_words;
   if (!part_pays(c, r)) return;
   // about 600 ranges of a perfect array (fewer leave SMs idle, more shorten the runs the scatter writes: 60M
   // rows in 391 ranges 334 us, in 1221 498 us), about 1024 of a hash table (smaller ranges spread hot keys),
   // of at least 256 slots, at most what an SM's shared memory holds
-  const int max_shift = hash ? 12 : words <= 1 ? 14 : 13;
+  const int max_shift = hash ? 12 : 14;
   int shift = 8;
   while (shift < max_shift && (g.cap >> shift) > (hash ? 1024 : 640)) ++shift;
   if (hash) shift = std::min(shift, g.log2cap);
@@ -727,11 +726,11 @@ static void alloc_part(pv_ctx* c, Result& r) {
   po.unit_rows = static_cast<uint32_t>(unit);
   const size_t n = (static_cast<size_t>(k.n_rows) + 3) & ~size_t(3);
   const size_t ctl = 4 * static_cast<size_t>(parts) + 2 + kPartCtlWords + kPartMaxRanges;
-  char* p = static_cast<char*>(dalloc(c, n * (8 * words + 4) + ctl * 4));
+  char* p = static_cast<char*>(dalloc(c, n * 12 + ctl * 4));
   if (!p) return;
   r.mem.push_back(p);
-  for (int w = 0; w < words; ++w, p += n * 8) po.val[w] = reinterpret_cast<unsigned long long*>(p);
-  po.key = reinterpret_cast<uint32_t*>(p);
+  po.val = reinterpret_cast<unsigned long long*>(p);
+  po.key = reinterpret_cast<uint32_t*>(p + n * 8);
   po.hist = po.key + n;
   po.done = po.hist + parts;
   po.ctl = po.done + parts;

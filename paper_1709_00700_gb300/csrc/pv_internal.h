@@ -179,14 +179,13 @@ struct GroupOut {
 // Scratch of the partitioned grouped aggregation (k_part.cuh), owned by a
 // result; key == nullptr: the result has none.  The words that start at zero
 // (clear_bytes from hist): rows per range, finished units per range, control.
-constexpr int kPartWords = 2;  // value words of a record at most
 enum { kPartCtlUnit = 0, kPartCtlDone = 1, kPartCtlFull = 2, kPartCtlWords = 4 };
 constexpr int kPartMaxRanges = 2048;
 constexpr int64_t kPartMinRows = 1 << 20;   // fewer rows: the general kernels
 constexpr int64_t kPartMinSlots = 1 << 12;  // of a perfect array
 struct PartOut {
   uint32_t* key;                        // records, by range: group key or slot
-  unsigned long long* val[kPartWords];  //   and aggregate codes
+  unsigned long long* val;              //   and value
   uint32_t* hist;                       // [n_parts] rows
   uint32_t* done;                       // [n_parts] units that added into the global table
   uint32_t* ctl;                        // next unit, finished CTAs of the count, a range was full
@@ -245,9 +244,9 @@ struct ShapeEntry {
   pv_status (*project)(const LaunchCfg&, const KParams&, const ProjOut&, int exec);
   pv_status (*grouped)(const LaunchCfg&, const KParams&, const GroupDesc&, const GroupOut&, const PartOut&,
                        const pv_variant&);
-  // grouped: value words of a partitioned record (-1: the shape has no
-  // partitioned kernels), and whether its hash tables have them too
-  int part_words;
+  // grouped: whether the shape's perfect arrays and hash tables have
+  // partitioned kernels
+  bool part_perfect;
   bool part_hash;
 };
 
