@@ -166,7 +166,8 @@ typedef enum { PV_GRID_STRIDE = 0, PV_CHUNKED = 1, PV_STAGED = 2 } pv_access;
 
 typedef struct {
   int32_t exec;              /* pv_exec: projection single pass (warp-aggregated atomics) or
-                                ordered by a prefix sum of match counts; aggregation: fused, or keys first */
+                                ordered by a prefix sum of match counts (compiled shapes then choose their
+                                own items_per_thread and access); aggregation: fused, or keys first */
   int32_t agg;               /* pv_agg_strategy for HASH_AGGREGATE */
   int32_t pred;              /* pv_pred_mode (all operations of the pipeline share it) */
   int32_t access;            /* pv_access: coalesced grid-stride, per-thread chunks, or TMA-staged chunks */
@@ -186,7 +187,7 @@ typedef struct {
   int32_t interp;            /* 0: the kernel compiled for the pipeline's shape when one exists, else the
                                 generic kernels; 1: always the generic kernels, which read the pipeline
                                 program (predicates, probes, key parts, aggregate terms, projected values)
-                                at run time, one row per thread.  The generic kernels implement the
+                                at run time.  The generic kernels implement the
                                 branched and predicated modes, grid-stride access, single and multi pass,
                                 and global or CTA-local tables; the other axes (chunked access, compacted
                                 mode, thread-private and cluster tables, warp pre-aggregation) return
@@ -264,7 +265,18 @@ pv_status pv_rebuild_hash_table(pv_ctx* ctx, pv_ht ht);
  * shape, or else on the generic kernels (see pv_variant.interp).  Limits that
  * return PV_ERR_UNSUPPORTED: more than 8 distinct fact columns; a group key of
  * three parts (or of two, one 64 bits wide) whose parts' value spans multiply
- * to more than 2^40; a variant axis the chosen kernels do not implement. */
+ * to more than 2^40; a variant axis the chosen kernels do not implement.
+ *
+ * HASH_AGGREGATE of one SUM and COUNTs over a million rows or more into global
+ * tables (PV_AGG_GLOBAL, single pass, perfect or linear, no probes) may be
+ * partitioned: rows are sorted by table range first.  That is decided from the
+ * column statistics, the table's size and a sample of the keys, for variants
+ * that the general kernels accept; block, grid_mult, items_per_thread, access,
+ * pred, prefetch and warp_agg then do not matter.  A result that may be
+ * partitioned holds 12 bytes of scratch per table row until it is freed, or
+ * until another allocation of the ctx fails: the scratch then goes back to the
+ * allocator (unless a captured graph refers to it) and the result runs on the
+ * general kernels, as it does when the scratch cannot be had at all. */
 pv_status pv_run_pipeline(pv_ctx* ctx, const pv_pipeline_spec* spec, const pv_variant* var,
                           pv_res* out);
 /* Enqueues the same pipeline again into the same result buffers (clearing
@@ -272,7 +284,9 @@ pv_status pv_run_pipeline(pv_ctx* ctx, const pv_pipeline_spec* spec, const pv_va
  * pv_graph_capture_begin/end. */
 pv_status pv_rerun(pv_ctx* ctx, pv_res res);
 /* Waits for the ctx stream (bounded by the watchdog, default 60 s) and
- * returns the first kernel-detected error since the last sync, clearing it. */
+ * returns the first kernel-detected error since the last sync, clearing it.
+ * The first 500 us of a wait are polled without sleeping, so that short queries
+ * return promptly: the calling thread keeps its core busy meanwhile. */
 pv_status pv_sync(pv_ctx* ctx);
 /* Watchdog limit of pv_sync in milliseconds (> 0). */
 pv_status pv_set_timeout_ms(pv_ctx* ctx, int64_t ms);

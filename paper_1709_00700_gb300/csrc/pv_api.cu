@@ -117,6 +117,8 @@ struct Result {
   GroupDesc gd{};
   GroupOut grp{};
   PartOut part{};
+  void* part_mem = nullptr;    // its scratch (one of mem)
+  bool part_captured = false;  // a graph's nodes refer to it
   int n_cols = 0;
   int col_type[PV_MAX_KEYS + PV_MAX_AGGS]{};
   int64_t rows_cached = -1;
@@ -173,7 +175,8 @@ pv_status cuda_fail(pv_ctx* c, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call); \
   } while (0)
 
-void* dalloc(pv_ctx* c, size_t bytes) {
+// Memory from the context's allocator, or null.
+void* try_alloc(pv_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 16;
   bytes = (bytes + 255) & ~size_t(255);
   if (c->alloc) return c->alloc(bytes, c->user);
@@ -189,6 +192,31 @@ void dfree(pv_ctx* c, void* p) {
   if (!p) return;
   if (c->free_) c->free_(p, c->user);
   else cudaFreeAsync(p, c->stream);
+}
+
+// Gives the scratch of the partitioned aggregations back to the allocator, except where a captured graph refers to
+// it; their results run on the general kernels from then on.  Returns whether there was any.
+bool give_back_scratch(pv_ctx* c) {
+  if (c->capturing) return false;
+  bool any = false;
+  for (auto& kv : c->results) {
+    Result& r = *kv.second;
+    if (!r.part_mem || r.part_captured) continue;
+    if (!any) cudaStreamSynchronize(c->stream);  // runs in flight use it
+    any = true;
+    r.mem.erase(std::find(r.mem.begin(), r.mem.end(), r.part_mem));
+    dfree(c, r.part_mem);
+    r.part_mem = nullptr;
+    r.part = PartOut{};
+  }
+  return any;
+}
+
+// Memory a call cannot do without: optional scratch gives way to it.
+void* dalloc(pv_ctx* c, size_t bytes) {
+  void* p = try_alloc(c, bytes);
+  if (!p && give_back_scratch(c)) p = try_alloc(c, bytes);
+  return p;
 }
 
 int type_size(int t) { return t == PV_I32 ? 4 : t == PV_I64 ? 8 : 1; }
@@ -726,9 +754,10 @@ static void alloc_part(pv_ctx* c, Result& r) {
   po.unit_rows = static_cast<uint32_t>(unit);
   const size_t n = (static_cast<size_t>(k.n_rows) + 3) & ~size_t(3);
   const size_t ctl = 4 * static_cast<size_t>(parts) + 2 + kPartCtlWords + kPartMaxRanges;
-  char* p = static_cast<char*>(dalloc(c, n * 12 + ctl * 4));
+  char* p = static_cast<char*>(try_alloc(c, n * 12 + ctl * 4));
   if (!p) return;
   r.mem.push_back(p);
+  r.part_mem = p;
   po.val = reinterpret_cast<unsigned long long*>(p);
   po.key = reinterpret_cast<uint32_t*>(p + n * 8);
   po.hist = po.key + n;
@@ -910,6 +939,11 @@ static pv_status launch_result(pv_ctx* c, Result& r) {
     if (k.mode == MODE_AGGREGATE) s = r.entry->aggregate(L, k.kp, r.agg);
     else if (k.mode == MODE_PROJECT) s = r.entry->project(L, k.kp, r.proj, r.var.exec);
     else s = r.entry->grouped(L, k.kp, r.gd, r.grp, r.part, r.var);
+    if (r.part_mem && !r.part_captured) {  // a graph captured here or by the caller keeps the scratch
+      cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+      r.part_captured = st != cudaStreamCaptureStatusNone;
+    }
   }
   if (s == PV_ERR_UNSUPPORTED) return fail(c, s, "no instantiation of this shape for the variant");
   if (s != PV_OK) return fail(c, s, "kernel launch failed");
