@@ -248,8 +248,8 @@ __device__ __forceinline__ void flush_out_rows(const char* st, int n, const Proj
 // sp_flush rows is staged in shared memory until that many are there: 15M
 // rows with 9% matching, 12 rows a trip, were bound by the cursor (118 us).
 // Output order is arbitrary across warps.  Trips of several items flush more
-// rows: at 64, 50M rows with 25% matching, 64 a trip of two items, took 280 us
-// against 235 without stages.
+// rows: 50M rows with 25% matching, 64 a trip of two items, took 235 us without
+// stages, 274 when flushed at 64 and 168 at 96.
 template <int U>
 constexpr int sp_flush() { return U == 1 ? 64 : 96; }
 template <int U>
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const __grid_constant__ Proj
 // lane, coalesced.  The filter runs once and the projected columns are read for
 // matching rows only: bound by the filter columns' bytes.  Filtering twice
 // around a scan kernel took 97 + 13 + 146 us for 50M rows with 2% matching (the
-// query with its result delivered 264 us, now 122 us).
+// query with its result delivered 264 us, now 111 us).
 // ---------------------------------------------------------------------------
 // The shape's filters and probes alone (no sink).
 template <class SH>
@@ -467,8 +467,7 @@ __global__ void __launch_bounds__(kMarkTileRows / 32) k_project_emit(const __gri
     }
     __syncthreads();  // the list is free again
   }
-  // The last CTA leaves the counters at zero for the next run: a clear ahead of the marks was a launch of its own
-  // (1M rows 12.3 us).
+  // The last CTA leaves the counters at zero for the next run: a clear ahead of the marks was a launch of its own.
   __shared__ bool last;
   if (threadIdx.x == 0) {
     __threadfence();
@@ -746,12 +745,10 @@ static pv_status launch_proj_sp(const LaunchCfg& c, const KParams& kp, const Pro
   return cudaGetLastError() == cudaSuccess ? PV_OK : PV_ERR_CUDA;
 }
 
-// Ordered projection.  The rows and their order do not depend on access and
-// items_per_thread, so the kernels choose both: the marks take 4 items a lane
+// The rows of an ordered projection and their order do not depend on access and
+// items_per_thread, so its kernels choose both: the marks take 4 items a lane
 // once that leaves an SM four warps with a unit each (10M rows, one filter,
-// 10% matching: 72 us with one item, 37 with four; 100K rows 6.9 / 8.2).  A
-// tile is split until an SM has three units, at most into 8 (100K rows, all
-// matching: 14 us by whole tiles, 8 by counting twice).
+// 10% matching: 72 us with one item, 37 with four; 100K rows 6.9 / 8.2).
 static bool mark_wide(const LaunchCfg& c, const KParams& kp) {
   return kp.n_items >= static_cast<int64_t>(512) * c.sm_count;
 }
@@ -767,6 +764,7 @@ static pv_status launch_proj_ordered(const LaunchCfg& c, const KParams& kp, cons
                           static_cast<int64_t>(c.block) * (wide ? 4 : 1));
   const int resident = grid_for(ce, reinterpret_cast<const void*>(ke), 0, INT32_MAX, 1);
   if (gm <= 0 || resident <= 0) return PV_ERR_UNSUPPORTED;
+  // until an SM has three units (100K rows, all matching: 14 us by whole tiles, 8 so)
   int split = 0;
   while (split < 3 && (mark_tiles(kp.n_rows) << split) < 3 * static_cast<int64_t>(c.sm_count)) ++split;
   const int ge = static_cast<int>(std::min<int64_t>(resident, mark_tiles(kp.n_rows) << split));

@@ -207,9 +207,11 @@ __device__ __forceinline__ void for_items_pf(const KParams& kp, F&& f) {
 // Branched grid-stride item loop (trips and items of for_items) that loads the
 // first column of a warp's next trip before it evaluates this one: the first
 // read of every trip is whole columns at DRAM latency, and the reads behind it
-// depend on it (Q5-shaped chain 428 -> 416 us; in the compacted loop the
-// registers it holds cost more than it gives, 163 -> 181 us for the star join).  f(items, idx) evaluates with FIRST.  All lanes of a warp run
-// every trip, items past the end empty.
+// depend on it (60M rows: lowcard grouping 638 -> 569 us, star join by branches
+// 206 -> 177, filter and two probes 273 -> 241; 1M rows, one or two trips: up
+// to 1 us slower.  In the compacted loop the registers it holds cost more than
+// it gives, 163 -> 181 us for the star join).  f(items, idx) evaluates with
+// FIRST.  All lanes of a warp run every trip, items past the end empty.
 template <class SH, int U, class F>
 __device__ __forceinline__ void for_items_ahead(const KParams& kp, F&& f) {
   constexpr int S = first_slot<SH>();

@@ -95,9 +95,8 @@ struct ProjOut {
   uint32_t* bits;
 };
 
-// Scratch of the ordered projection: a tile is 256 bitmap words, a super a group of tiles: 16, which
-// spreads the marks' counters (one super for 64 tiles took 12 us instead of 9 for 1M rows), or as many as
-// leave 2048 supers to add up.
+// Scratch of the ordered projection: a tile is 256 bitmap words, a super a group of tiles: 16, so that few
+// warps of the marks meet on its counter, or as many as leave 2048 supers to add up.
 constexpr int kMarkTileRows = 8192;
 __host__ __device__ inline int64_t mark_tiles(int64_t n_rows) {
   return n_rows > kMarkTileRows ? (n_rows + kMarkTileRows - 1) / kMarkTileRows : 1;
