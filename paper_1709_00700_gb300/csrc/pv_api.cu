@@ -698,28 +698,40 @@ static bool part_pays(pv_ctx* c, const Result& r) {
   for (int i = 0; i < k.n_keys; ++i) hot_share *= static_cast<double>(c->cols[k.key_src[i][0]].top) / kSampleRows;
   const bool hot = hot_share >= 1.0 / 64;
   const int64_t bytes = g.cap * (g.stride + (hash ? 1 : 0)) * 8;
-  const bool large = bytes >= (int64_t(16) << 20), far = bytes > c->l2_bytes;
+  const bool large = bytes >= (int64_t(16) << 20), mid = bytes >= (int64_t(48) << 20), far = bytes > c->l2_bytes;
   const int64_t M = int64_t(1) << 20;
+  const double kept = keep * static_cast<double>(n);
   if (hash) {
-    // 300K and 1M groups: all of 1.1M uniform rows 62 / 56, 102 / 62, 30% 59 / 59, 81 / 62, 10% 44 / 57, 59 / 60
-    if (n < 4 * M) return large && keep >= 0.3;
-    if (hot) return keep >= (n < 16 * M ? 0.3 : 0.01);  // 4.3M rows, 30K groups: 30% 174 / 101, 10% 85 / 94
-    // 4.3M uniform rows, 300K groups: 30% 127 / 97, 90% 128 / 133, all 119 / 131; 1M groups all 215 / 147
-    if (n < 16 * M) return large && keep >= 0.3 && (filtered || bytes >= (int64_t(48) << 20));
-    // 60M uniform rows: 300K groups 1% 1000 / 432, 30% 1382 / 835, 90% 1445 / 1323, all 1092 / 1113; all of 1000
-    // groups 2125 / 1580
-    return filtered ? keep >= 0.01 : far || g.cap <= (int64_t(1) << 12);
+    // 300K groups, uniform: 1.1M rows 10% 44 / 57, 30% 59 / 59; 2M rows 10% 66 / 61, 20% 78 / 62
+    if (n < 4 * M) return large && kept >= 250e3;
+    // skewed, 30K groups: 4.3M rows 10% 85 / 94, 30% 174 / 101; 13M rows 3% 187 / 200, 10% 270 / 235; 17M rows 1%
+    // 192 / 151; 30M rows 0.3% 244 / 186
+    const double least = n < 5 * M ? 0.12 : n < 12 * M ? 0.1 : n < 16 * M ? 0.03 : n < 24 * M ? 0.01 : 0.003;
+    if (hot) return keep >= (large && n >= 8 * M ? std::min(least, 0.03) : least);  // 300K groups 9M rows 3% 153 / 146
+    // uniform, 300K groups: 6M rows 20% 163 / 120, 90% 178 / 180, all 157 / 163; 1M groups all 262 / 197, all of 60M
+    // 1630 / 1783
+    if (large && filtered) return keep >= (n >= 8 * M ? std::min(least, 0.03) : least);  // 9M rows 3% 172 / 128
+    if (large) return far || (mid && n < 16 * M);
+    // uniform, few groups: 1000, all of 4.3M rows 184 / 155; 30K, 9M rows 10% 154 / 144, 50% 260 / 233, 90% 274 / 287,
+    // all 230 / 256; 13M rows 3% 201 / 146, 90% 407 / 390
+    if (!filtered) return g.cap <= (int64_t(1) << 12);
+    return n >= 8 * M && (n >= 12 * M ? keep >= least : keep >= 0.2 && keep < 0.8);
   }
-  // 60M rows, 1e7 groups, far: all 2342 / 650, 30% 967 / 743, 10% 547 / 641; three key parts, 9.3M slots 2407 / 1091
-  if (far && keep >= 0.2) return true;
-  // skewed keys: all of 1.1M rows, 4200 groups 164 / 34; 30% of 1.1M rows, 1e5 groups 74 / 40, 10% 31 / 38; 10% of
-  // 4.3M rows 96 / 63; 1% of 60M rows 253 / 415
-  if (hot && keep >= (n < 4 * M ? 0.3 : 0.1)) return true;
-  // few slots and many rows, which collide: 17M rows, 4200 groups 394 / 178, 90% 359 / 263, 30% 137 / 194; 1e4
-  // groups 242 / 178, 90% 220 / 263; three key parts, 4913 slots 348 / 282, 216K slots 207 / 317
-  if (n >= 16 * M && g.cap <= (filtered ? int64_t(1) << 13 : int64_t(1) << 14) && keep >= 0.8) return true;
-  // a large table in L2: 1e6 groups, all of 1.1M rows 42 / 34, of 60M 672 / 641, 90% of 60M 620 / 956; three key
-  // parts, 60M rows, 2.2M slots 772 / 1111
+  // 1e7 groups, far: 3% of 8M rows 171 / 132, all 544 / 156; 10% of 30M 394 / 362; 60M rows 10% 547 / 641, 30%
+  // 967 / 743; three key parts, 9.3M slots, all of 60M 2407 / 1091
+  if (far && keep >= (n < 16 * M ? 0.03 : n < 48 * M ? 0.1 : 0.2)) return true;
+  // skewed: all of 1.1M rows, 4200 groups 164 / 34; 2M rows, 1e5 groups 10% 49 / 43, 3% 21 / 41; 8M rows 10%
+  // 172 / 111, 3% 62 / 95; 60M rows 1% 253 / 415
+  if (hot && keep >= 0.08 && kept >= 180e3) return true;
+  // few slots and many rows, which collide: 4200 groups, all of 4.3M rows 102 / 66; 1e4, all of 4.3M 66 / 66, of 17M
+  // 242 / 178; 2e4, all of 30M 371 / 300; 4200, 90% of 17M 359 / 263, 30% 137 / 194; three key parts, 4913 slots,
+  // all of 17M 348 / 282, 216K slots 207 / 317
+  const int64_t few = filtered ? (n >= 16 * M && keep >= 0.8 ? 8 : 0) : n < 4 * M ? 0 : n < 16 * M ? 8 : n < 24 * M ? 16 : 32;
+  if (g.cap <= few << 10) return true;
+  // a table of some size in L2 and few rows: 3M groups, 10% of 2M rows 73 / 50, of 8M 112 / 120
+  if (mid && n < 4 * M && keep >= 0.1) return true;
+  // 1e6 groups, all of 1.1M rows 42 / 34, of 60M 672 / 641, 90% of 60M 620 / 956; three key parts, 2.2M slots, all of
+  // 60M 772 / 1111
   return large && !filtered && k.n_keys == 1;
 }
 

@@ -38,9 +38,10 @@ M = 1 << 20
 @pytest.mark.parametrize("n,groups,skew,keep,part", [
     (M - 1, 9_000_000, True, None, False), (M, 9_000_000, False, None, True), (M, 4_095, True, None, False),
     (M, 4_096, True, None, True), (M, 4_096, False, None, False), (M, 50_000, True, 0.35, True),
-    (M, 50_000, True, 0.2, False), (M, 50_000, False, 0.9, False), (4 * M + 5, 50_000, True, 0.15, True),
+    (M, 50_000, True, 0.1, False), (M, 50_000, False, 0.9, False), (4 * M + 5, 50_000, True, 0.15, True),
     (4 * M + 5, 50_000, True, 0.05, False), (M + 3, 1_000_000, False, None, True),
-    (M + 3, 1_000_000, False, 0.9, False), (M + 3, 9_000_000, False, 0.25, True), (M + 3, 9_000_000, False, 0.15, False),
+    (M + 3, 1_000_000, False, 0.9, False), (M + 3, 9_000_000, False, 0.1, True), (M + 3, 9_000_000, False, 0.02, False),
+    (2 * M, 3_000_000, False, 0.2, True), (4 * M - 1, 5_000, False, None, False), (4 * M, 5_000, False, None, True),
     (16 * M, 9_999, False, None, True), (16 * M, 60_000, False, None, False), (16 * M + 9, 5_000, False, 0.9, True),
     (16 * M + 9, 5_000, False, 0.5, False)])
 def test_perfect(n, groups, skew, keep, part):
@@ -63,6 +64,7 @@ def test_perfect(n, groups, skew, keep, part):
     (M, 600_000, False, 0.5, True), (M, 600_000, False, 0.2, False), (M, 60_000, True, 0.9, False),
     (4 * M, 60_000, True, 0.5, True), (4 * M, 60_000, True, 0.1, False), (4 * M, 60_000, False, 0.9, False),
     (4 * M, 300_000, False, 0.5, True), (4 * M, 300_000, False, None, False), (4 * M, 900_000, False, None, True),
+    (4 * M, 2_000, False, None, True), (9 * M, 60_000, False, 0.5, True), (9 * M, 60_000, False, 0.9, False),
     (16 * M, 2_000, False, None, True), (16 * M, 60_000, False, None, False), (16 * M, 60_000, False, 0.02, True),
     (16 * M, 60_000, False, 0.005, False)])
 def test_linear(n, groups, skew, keep, part):
